@@ -92,6 +92,12 @@ def step_launches(steps, mid_per_step, fused):
     return chunks * seq(32) + sum(seq(1 << b) for b in range(5) if rem >> b & 1)
 
 
+def line_launches(steps):
+    """Launches of the 1-D cooperative stepping kernel for one `step` call (at most 65536 steps a launch); the
+    1-D workloads fit its shared memory."""
+    return -(-steps // 65536)
+
+
 def fused_in_steps(spec: dict, shapes: dict, option: int = 0) -> bool:
     """Whether the timed steps run the fused E + H pass: asked for by option
     (2-D / 3-D FP32), or chosen by the autotuner (2-D FP32, fused_rows > 0)."""
@@ -355,7 +361,8 @@ def solver_config(workload: str, steps: int, warmup: int, autotune: bool, local:
                          "traffic": ncu_traffic(kname, workload, kshape),
                          "peak_source": src},
             "step_hbm_frac_algorithmic": step_alg / (ms_step / 1e3) / 1e9 / peak,
-            "gpu_launches": step_launches(steps, 1 if ns else 0, fused_in_steps(spec, shapes))}
+            "gpu_launches": (line_launches(steps) if spec["grid"]["ndim"] == 1 else
+                             step_launches(steps, 1 if ns else 0, fused_in_steps(spec, shapes)))}
 
 
 def batch_config(workload: str, specs, steps: int, warmup: int, autotune: bool, local: int) -> dict:
@@ -770,7 +777,8 @@ def main():
             "stencil_ms_in_step": ms_step - kt["kinetic"] - kt["closure"],
             "launch_shapes": dict(shapes, tuned=tune is not None),
             "roofline": roof,
-            "gpu_launches": step_launches(args.steps, 1 if ns else 0, fused),
+            "gpu_launches": (line_launches(args.steps) if spec["grid"]["ndim"] == 1 else
+                             step_launches(args.steps, 1 if ns else 0, fused)),
             "clocks": clk,
             "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d / args.steps,
                     "d2h_bytes_per_step": d2h / args.steps, "breakdown_ms": e2e_breakdown_ms}}

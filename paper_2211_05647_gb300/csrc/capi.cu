@@ -5,6 +5,7 @@
 //
 // Every coefficient is derived here from the paper's formulas, in FP64 on the
 // host, then rounded once to the field precision.
+#include <algorithm>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -21,6 +22,7 @@
 #include <nvtx3/nvToolsExt.h>
 
 #include "internal.cuh"
+#include "line1d.cuh"
 
 using namespace fp;
 
@@ -171,8 +173,18 @@ bool pol_updated(const fdtd_plasma *h, int64_t c)
     return j >= 1 && k >= 1;
 }
 
+// the 1-D stepping kernel's plan follows the slot layout: made again on the next step
+void free_line(fdtd_plasma *h)
+{
+    dfree(h, h->line_cut); dfree(h, h->line_mail);
+    h->line_cut = nullptr;
+    h->line_mail = nullptr;
+    h->line_state = 0;
+}
+
 void free_closure(fdtd_plasma *h)
 {
+    free_line(h);
     dfree(h, h->hist); dfree(h, h->jprev); dfree(h, h->params);
     h->hist = h->jprev = h->params = nullptr;
     h->has_closure = 0;
@@ -739,6 +751,108 @@ cudaError_t enqueue(fdtd_plasma *h, cudaStream_t st, int nsteps)
     if (e != cudaSuccess) return e;
     launch_advance(st, h->d_step, nsteps);
     return cudaGetLastError();
+}
+
+// ------------------------------------------------- 1-D: many steps a launch
+// A 1-D grid whose state fits in the SMs' shared memory (E, H and the linear delta-f rows, one equal-cost range
+// per SM; rows of up to 128 sixteen-byte vectors) steps through the cooperative kernel of line1d.cu; what reads
+// or adds to a step from outside (ports, the recorder, the closure) and the nonlinear and evolving-F0 rows take
+// the step graphs.  Measured against the graphs over the sizes that fit: 500 rows of 64 nodes on 2000 cells, FP32
+// 0.97 against 6.0 us a step, FP64 2.3 against 13.1; 30 k rows, FP32 4.9 against 8.0; 100 k BF16 rows 11.6 both
+// (FP32: no longer fits); a million cells without plasma 2.6 against 8.7.  So what fits takes the kernel.
+bool line_applies(const fdtd_plasma *h)
+{
+    if (h->g.ndim != 1 || h->nports > 0 || h->has_recording || h->has_closure) return false;
+    return !(h->has_plasma && (h->pl.nonlinear || h->pl.evolve_f0));
+}
+
+int line_plan(fdtd_plasma *h)
+{
+    h->line_state = -1;
+    const int f_dtype = h->g.precision == FDTD_F64 ? FDTD_DF_F64 : (h->has_plasma ? h->pl.f_dtype : FDTD_DF_F32);
+    const int pitch = h->has_plasma ? h->pitch : 0, vec = f_dtype == FDTD_DF_BF16 ? 8 : (f_dtype == FDTD_DF_F64 ? 2 : 4);
+    if (pitch / vec > 128) return FDTD_OK;
+    // a row weighs its nodes: an FP64 row is bound by the FP64 pipe, and the cells of a range cost next to nothing
+    const LinePlan p = line1d_plan(h->nz, h->h_cells, h->num_sms, (double)pitch);
+    int dev = 0, most = 0;
+    CK(h, cudaGetDevice(&dev));
+    CK(h, cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
+    if (line1d_smem_bytes(f_dtype, pitch, p.rows_max, p.nodes_max) + 1024 > (size_t)most) return FDTD_OK;
+    const size_t n = p.cut.size();
+    h->line_cut = (int32_t *)dalloc(h, 2 * n * sizeof(int32_t));
+    h->line_mail = (uint64_t *)dalloc(h, (n - 1) * 8 * sizeof(uint64_t));
+    if (!h->line_cut || !h->line_mail) {   // no room: the graphs need none of it
+        free_line(h);
+        h->err.clear();
+        h->line_state = -1;
+        return FDTD_OK;
+    }
+    std::vector<int32_t> both(p.cut);
+    both.insert(both.end(), p.slot_cut.begin(), p.slot_cut.end());
+    CK(h, cudaMemsetAsync(h->line_mail, 0, (n - 1) * 8 * sizeof(uint64_t), h->stream));
+    CK(h, cudaMemcpyAsync(h->line_cut, both.data(), both.size() * sizeof(int32_t), cudaMemcpyHostToDevice, h->stream));
+    CK(h, cudaStreamSynchronize(h->stream));
+    h->line_ctas = (int)n - 1;
+    h->line_rows = p.rows_max;
+    h->line_nodes = p.nodes_max;
+    h->line_seq = 1;
+    h->line_state = 1;
+    return FDTD_OK;
+}
+
+template <typename T>
+cudaError_t line_launch(fdtd_plasma *h, int nsteps)
+{
+    const double mu0 = 1.0 / (kEps0 * kC0 * kC0);
+    LineArgs<T> a{};
+    a.E = reinterpret_cast<T *>(h->f[FDTD_EX]);
+    a.H = reinterpret_cast<T *>(h->f[FDTD_HY]);
+    a.mur = h->g.mur ? reinterpret_cast<T *>(h->mur_state) : nullptr;
+    a.cut = h->line_cut;
+    a.slot_cut = h->line_cut + h->line_ctas + 1;
+    if (h->has_plasma) {
+        a.jslot = reinterpret_cast<T *>(h->jslot);
+        a.df = h->df;
+        a.dens = reinterpret_cast<const T *>(h->dens);
+        a.tab = reinterpret_cast<const T *>(h->tab);
+        a.slot_cell = h->slot_cell;
+        a.pitch = h->pitch;
+        a.seed = h->pl.seed;
+    }
+    a.mail = h->line_mail;
+    a.d_step = h->d_step;
+    a.err = h->d_err;
+    a.src = source_view(h);
+    a.step0 = h->steps_done;
+    a.seq = h->line_seq;
+    a.nsteps = nsteps;
+    a.nz = (int)h->nz;
+    a.rows_max = h->line_rows;
+    a.nodes_max = h->line_nodes;
+    a.ch = (T)(h->dt / (mu0 * h->g.dx));
+    a.ce = (T)(h->dt / (kEps0 * h->g.dx));
+    a.cj = (T)(h->dt / kEps0);
+    a.m = (T)((kC0 * h->dt - h->g.dx) / (kC0 * h->dt + h->g.dx));
+    return launch_line1d<T>(h->stream, a, h->has_plasma ? h->pl.f_dtype : (sizeof(T) == 8 ? FDTD_DF_F64 : FDTD_DF_F32),
+                            h->line_ctas);
+}
+
+int line_step(fdtd_plasma *h, int64_t nsteps)
+{
+    // the launch carries the step and message counters as arguments: it is not for replay in a caller's graph
+    // (the step graphs cannot be captured either)
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    CK(h, cudaStreamIsCapturing(h->stream, &cs));
+    if (cs != cudaStreamCaptureStatusNone) return cuda_fail(h, cudaErrorStreamCaptureUnsupported, "fdtd_plasma_step");
+    for (int64_t left = nsteps; left > 0;) {
+        const int n = (int)std::min<int64_t>(left, 65536);
+        const cudaError_t e = h->g.precision == FDTD_F64 ? line_launch<double>(h, n) : line_launch<float>(h, n);
+        if (e != cudaSuccess) return cuda_fail(h, e, "1-D stepping kernel");
+        h->line_seq += (uint32_t)n;
+        h->steps_done += n;
+        left -= n;
+    }
+    return FDTD_OK;
 }
 
 int capture(fdtd_plasma *h, int nsteps, cudaGraphExec_t *out)
@@ -1339,6 +1453,13 @@ int fdtd_plasma_step(fdtd_plasma_t h, int64_t nsteps)
     if (h->sd_on && (h->sd_lo || h->sd_hi || h->sd_half))
         return fail(h, FDTD_ERR_STATE, "a sub-domain with neighbours steps by fdtd_plasma_step_half, exchanging halos");
     if (nsteps == 0) return FDTD_OK;
+    if (line_applies(h)) {
+        if (h->line_state == 0) {
+            const int rc = line_plan(h);
+            if (rc != FDTD_OK) return rc;
+        }
+        if (h->line_state > 0) return line_step(h, nsteps);
+    }
     if (!h->graphs_valid) {
         ensure_second_set(h);
         int rc = capture(h, 1, &h->g1);
@@ -1820,9 +1941,10 @@ size_t fdtd_plasma_quantity_bytes(fdtd_plasma_t h, int which)
     return 0;
 }
 
-// the device error word: bit 1 closure tensor-core waits, bit 2 TMA stencil waits
+// the device error word: bit 1 closure tensor-core waits, bit 2 TMA stencil waits, bit 4 1-D neighbour waits
 static const char *wait_error_text(int errw)
 {
+    if (errw & 4) return "a bounded device wait gave up (1-D stepping kernel)";
     if (errw & 2) return "a bounded device wait gave up (TMA stencil kernel)";
     return "a bounded device wait gave up (closure kernel)";
 }

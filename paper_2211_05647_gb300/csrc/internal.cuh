@@ -142,6 +142,17 @@ __device__ __forceinline__ void two_sum(T a, T b, T &s, T &e)
     T z = s - a;
     e = (a - (s - z)) + (b - z);
 }
+// FP64 on sm_103a: every FP64 instruction holds its sub-core's pipe for 64 cycles, whatever the number of active
+// lanes (measured with dependent and independent chains, 1 to 16 warps).  Dekker's three-operation form gives
+// the same s and e when a's exponent is not below b's; the ordering is two integer operations and four selects.
+template <>
+__device__ __forceinline__ void two_sum<double>(double a, double b, double &s, double &e)
+{
+    const bool ab = (__double2hiint(a) & 0x7fffffff) >= (__double2hiint(b) & 0x7fffffff);
+    const double hi = ab ? a : b, lo = ab ? b : a;
+    s = hi + lo;
+    e = lo - (s - hi);
+}
 
 // ------------------------------------------- Philox4x32-7 (Salmon et al. 2011)
 // The 7-round variant, which the authors report passes TestU01's BigCrush;
@@ -450,6 +461,12 @@ struct fdtd_plasma {
     cudaGraphExec_t gpow[4];   // 2-, 4-, 8- and 16-step graphs for a call's remainder (captured on first use)
     int gk_steps;
     int graphs_valid;
+    // the 1-D cooperative stepping kernel (line1d.cu): ranges and mailboxes, made on the first step
+    // (line_state 0: not looked at yet, 1: in use, -1: this configuration takes the step graphs)
+    int line_state, line_ctas, line_rows, line_nodes;
+    uint32_t line_seq;         // tag of the next launch's first message
+    int32_t *line_cut;         // cut[line_ctas + 1], then slot_cut[line_ctas + 1]
+    uint64_t *line_mail;
     // running-DFT ports (device arrays; nports = 0: none)
     int nports, nfreq;
     int64_t *port_off, *port_cells;

@@ -76,20 +76,26 @@ __device__ __forceinline__ void lds(const double *p, double *x)
     }
 }
 
+// pack: compute values -> a storage vector; st: the same, stored to global memory (streaming)
 template <typename TS>
 struct Store;
 template <>
 struct Store<float> {
-    static __device__ __forceinline__ void st(float4 *p, const float *x, uint4, uint2)
+    static __device__ __forceinline__ float4 pack(const float *x, uint4, uint2)
     {
-        __stcs(p, make_float4(x[0], x[1], x[2], x[3]));
+        return make_float4(x[0], x[1], x[2], x[3]);
+    }
+    static __device__ __forceinline__ void st(float4 *p, const float *x, uint4 ctr, uint2 key)
+    {
+        __stcs(p, pack(x, ctr, key));
     }
 };
 template <>
 struct Store<double> {
-    static __device__ __forceinline__ void st(double2 *p, const double *x, uint4, uint2)
+    static __device__ __forceinline__ double2 pack(const double *x, uint4, uint2) { return make_double2(x[0], x[1]); }
+    static __device__ __forceinline__ void st(double2 *p, const double *x, uint4 ctr, uint2 key)
     {
-        __stcs(p, make_double2(x[0], x[1]));
+        __stcs(p, pack(x, ctr, key));
     }
 };
 // BF16 storage: one Philox4x32-7 call per 8 nodes (16 bits a node).  A vector
@@ -99,7 +105,7 @@ struct Store<double> {
 // through f32_to_bf16_sr, which keeps infinities and NaNs.
 template <>
 struct Store<__nv_bfloat16> {
-    static __device__ __forceinline__ void st(uint4 *p, const float *x, uint4 ctr, uint2 key)
+    static __device__ __forceinline__ uint4 pack(const float *x, uint4 ctr, uint2 key)
     {
         const uint4 r = philox4x32_7(ctr, key);
         const uint32_t rr[4] = {r.x, r.y, r.z, r.w};
@@ -118,12 +124,16 @@ struct Store<__nv_bfloat16> {
                 w[q] = lo | (hi << 16);
             }
         }
-        __stcs(p, make_uint4(w[0], w[1], w[2], w[3]));
+        return make_uint4(w[0], w[1], w[2], w[3]);
+    }
+    static __device__ __forceinline__ void st(uint4 *p, const float *x, uint4 ctr, uint2 key)
+    {
+        __stcs(p, pack(x, ctr, key));
     }
 };
 
 // One lane's share of a delta-f row: VPL vectors at indices q*L + l.  Updates
-// df <- alpha df + beta nE in place (store through Store<TS>) and returns the
+// df <- alpha df + beta nE (each new vector handed to put(index, vector)) and returns the
 // lane's partial sum of w' df in (s, c): compensated (TwoSum) for FP32 / FP64
 // rows; for BF16 rows a plain FP32 accumulation, whose rounding (~1e-6 of the
 // sum for a row of <= 1024 nodes) is far below the 2^-8 storage rounding of the
@@ -131,10 +141,10 @@ struct Store<__nv_bfloat16> {
 // the two-lane FP32 instructions: node pairs (2t, 2t+1) get alpha df + (beta nE)
 // with the roundings of the scalar fma, and the sum is kept as two partial sums
 // (even and odd nodes) added at the end.
-template <typename TS, typename TA, int VPL, int L>
-__device__ __forceinline__ void row_update(typename Vec<TS>::type *rp, const typename Vec<TS>::type *v,
-                                           const TA *al_tab, const TA *be_tab, const TA *w_tab, TA nE, int l,
-                                           uint32_t row_id, int64_t step, uint2 key, TA &s, TA &c)
+template <typename TS, typename TA, int VPL, int L, typename Put>
+__device__ __forceinline__ void row_update_to(const typename Vec<TS>::type *v, const TA *al_tab, const TA *be_tab,
+                                              const TA *w_tab, TA nE, int l, uint32_t row_id, int64_t step, uint2 key,
+                                              TA &s, TA &c, Put &&put)
 {
     constexpr int VEC = Vec<TS>::n;
     if constexpr (std::is_same<TS, __nv_bfloat16>::value) {
@@ -157,10 +167,11 @@ __device__ __forceinline__ void row_update(typename Vec<TS>::type *rp, const typ
                 x[t + 1] = xs.y;
             }
             const uint4 ctr = make_uint4(row_id, (uint32_t)vi, (uint32_t)step, (uint32_t)(step >> 32));
-            Store<TS>::st(rp + vi, x, ctr, key);
+            put(vi, Store<TS>::pack(x, ctr, key));
         }
         const float2 ss = f2_split(s2);
-        s += ss.x + ss.y;
+        s = ss.x + ss.y;
+        c = TA(0);
     } else {
 #pragma unroll
         for (int q = 0; q < VPL; ++q) {
@@ -173,14 +184,30 @@ __device__ __forceinline__ void row_update(typename Vec<TS>::type *rp, const typ
 #pragma unroll
             for (int t = 0; t < VEC; ++t) {
                 x[t] = al[t] * x[t] + be[t] * nE;
+                const TA p = mul_rn(w[t], x[t]);
+                if (q == 0 && t == 0) {   // the first term starts the sum
+                    s = p;
+                    c = TA(0);
+                    continue;
+                }
                 TA hi, lo;
-                two_sum(s, mul_rn(w[t], x[t]), hi, lo);
+                two_sum(s, p, hi, lo);
                 s = hi;
                 c += lo;
             }
-            Store<TS>::st(rp + vi, x, uint4{}, uint2{});
+            put(vi, Store<TS>::pack(x, uint4{}, uint2{}));
         }
     }
+}
+
+// the same in place on a row in global memory (streaming stores)
+template <typename TS, typename TA, int VPL, int L>
+__device__ __forceinline__ void row_update(typename Vec<TS>::type *rp, const typename Vec<TS>::type *v,
+                                           const TA *al_tab, const TA *be_tab, const TA *w_tab, TA nE, int l,
+                                           uint32_t row_id, int64_t step, uint2 key, TA &s, TA &c)
+{
+    row_update_to<TS, TA, VPL, L>(v, al_tab, be_tab, w_tab, nE, l, row_id, step, key, s, c,
+                                  [&](int vi, const typename Vec<TS>::type &x) { __stcs(rp + vi, x); });
 }
 
 // TwoSum tree over the L lanes sharing a row (xor offsets < L stay inside the group)
