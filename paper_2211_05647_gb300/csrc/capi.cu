@@ -1960,10 +1960,7 @@ static int copy_quantity(fdtd_plasma_t h, int which, void *host_or_dev, size_t b
     if (which == FDTD_DF || which == FDTD_F0) {
         void *rows = which == FDTD_DF ? h->df : h->g0;
         const size_t row = (size_t)h->nnode * h->df_esz, dpitch = (size_t)h->pitch * h->df_esz;
-        if (out)
-            CK(h, cudaMemcpy2DAsync(host_or_dev, row, rows, dpitch, row, h->nkin, kind, h->stream));
-        else
-            CK(h, cudaMemcpy2DAsync(rows, dpitch, host_or_dev, row, row, h->nkin, kind, h->stream));
+        CK(h, copy_rows(h->stream, host_or_dev, rows, h->nkin, row, dpitch, kind, out));
     } else {
         void *dev = which == FDTD_J ? h->jslot : h->f[which];
         if (out) CK(h, cudaMemcpyAsync(host_or_dev, dev, bytes, kind, h->stream));
