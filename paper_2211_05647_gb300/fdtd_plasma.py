@@ -691,21 +691,20 @@ class Solver:
         """Quantity as a torch tensor on the device (stream-ordered) or, with
         device=False, as a host numpy array (synchronous)."""
         torch = self.torch
-        nb = self.quantity_bytes(name)
+        lib, q = self.lib, QUANTITY[name]
+        nb = lib.fdtd_plasma_quantity_bytes(self.h, q)
+        rows = name in ("df", "f0")
         dt = self._dtype(name)
-        n = nb // torch.empty((), dtype=dt).element_size()
+        dev = self.device if device else "cpu"
         if nb == 0:     # no plasma (J, delta f) on this grid or sub-domain
-            out = torch.empty((0, self.plasma_shape()[1]) if name in ("df", "f0") else 0, dtype=dt,
-                              device=self.device if device else "cpu")
-            return out if device else (out.float().numpy() if dt == torch.bfloat16 else out.numpy())
-        if device:
-            out = torch.empty(n, dtype=dt, device=self.device)
-            _check(self.lib, self.h, self.lib.fdtd_plasma_read_fields(self.h, QUANTITY[name], out.data_ptr(), nb, 1))
+            out = torch.empty((0, self.plasma_shape()[1]) if rows else 0, dtype=dt, device=dev)
         else:
-            out = torch.empty(n, dtype=dt)
-            _check(self.lib, self.h, self.lib.fdtd_plasma_read_fields(self.h, QUANTITY[name], out.data_ptr(), nb, 0))
-        if name in ("df", "f0"):
-            out = out.view(self.plasma_shape())
+            out = torch.empty(nb // dt.itemsize, dtype=dt, device=dev)
+            rc = lib.fdtd_plasma_read_fields(self.h, q, out.data_ptr(), nb, 1 if device else 0)
+            if rc != FDTD_OK:
+                _check(lib, self.h, rc)
+            if rows:
+                out = out.view(self.plasma_shape())
         return out if device else (out.float().numpy() if dt == torch.bfloat16 else out.numpy())
 
     def write(self, name: str, values):
