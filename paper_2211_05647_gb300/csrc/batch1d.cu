@@ -664,7 +664,7 @@ int fdtd_batch_create(const fdtd_run_desc *runs, int32_t nruns, const fdtd_runti
     const std::vector<double> &w = vt.w, &f0p = vt.f0p;
     const int P = b->pitch;
     std::vector<double> tab((size_t)P * (1 + 2 * (size_t)nruns), 0.0);
-    for (int j = 0; j < nnode; ++j) tab[j] = -kQe * w[j];
+    for (int j = 0; j < nnode; ++j) tab[tab_pos(j, P, p0.f_dtype)] = -kQe * w[j];
     double wpmax = 0;
     // ---- per-run layout and slots
     std::vector<BRun> hr(nruns);
@@ -701,8 +701,9 @@ int fdtd_batch_create(const fdtd_run_desc *runs, int32_t nruns, const fdtd_runti
         const double nu0 = p.nu0;
         for (int j = 0; j < nnode; ++j) {
             const double nu = node_nu(p, vt, (size_t)j, nu0);
-            tab[(size_t)P * (1 + 2 * r) + j] = (2 - b->dt * nu) / (2 + b->dt * nu);
-            tab[(size_t)P * (2 + 2 * r) + j] = 2 * b->dt * (kQe / kMe) * f0p[j] / (2 + b->dt * nu);
+            const size_t q = tab_pos(j, P, p0.f_dtype);
+            tab[(size_t)P * (1 + 2 * r) + q] = (2 - b->dt * nu) / (2 + b->dt * nu);
+            tab[(size_t)P * (2 + 2 * r) + q] = 2 * b->dt * (kQe / kMe) * f0p[j] / (2 + b->dt * nu);
         }
         BRun &br = hr[r];
         br.e_off = eo; br.h_off = ho; br.row_off = ro;
@@ -908,8 +909,7 @@ int fdtd_batch_read(fdtd_batch_t b, int32_t run, int which, void *dst, size_t by
     cudaError_t e;
     if (which == FDTD_DF) {
         const size_t row = (size_t)b->nnode * b->df_esz, dp = (size_t)b->pitch * b->df_esz;
-        e = cudaMemcpy2DAsync(dst, row, (char *)b->df + b->row_off[run] * dp, dp, row, b->nslot[run], kind,
-                              b->stream);
+        e = copy_rows(b->stream, dst, (char *)b->df + b->row_off[run] * dp, b->nslot[run], row, dp, kind, true);
     } else {
         const char *src = which == FDTD_EX   ? (char *)b->E + b->e_off[run] * b->esz
                           : which == FDTD_HY ? (char *)b->H + b->h_off[run] * b->esz

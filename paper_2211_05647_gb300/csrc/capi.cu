@@ -1336,9 +1336,10 @@ int fdtd_plasma_set_plasma(fdtd_plasma_t h, const fdtd_plasma_desc *p)
     std::vector<double> tab(3 * (size_t)pitch, 0.0);
     for (int64_t j = 0; j < nnode; ++j) {
         const double nu = t.nu[j];
-        tab[j] = (2.0 - h->dt * nu) / (2.0 + h->dt * nu);
-        tab[pitch + j] = 2.0 * h->dt * (kQe / kMe) * t.f0p[j] / (2.0 + h->dt * nu);
-        tab[2 * pitch + j] = -kQe * t.w[j];
+        const size_t q = tab_pos((size_t)j, (size_t)pitch, p->f_dtype);
+        tab[q] = (2.0 - h->dt * nu) / (2.0 + h->dt * nu);
+        tab[pitch + q] = 2.0 * h->dt * (kQe / kMe) * t.f0p[j] / (2.0 + h->dt * nu);
+        tab[2 * pitch + q] = -kQe * t.w[j];
     }
     // evolve_f0 tables (padding 0): f0, f0', bq = 2 dt (e/m) / (2 + dt nu), v^3, 1/(v^2 gam), and for
     // the upper cell edge v_e = (j+1) gam of each node but the last: 1/(2 v_e), (m/M) v_e^3 nu_e

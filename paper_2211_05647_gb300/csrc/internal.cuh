@@ -291,8 +291,15 @@ cudaError_t copy_rows(cudaStream_t st, void *packed, void *padded, int64_t rows,
 
 // delta-f row pitch (elements) for nnode nodes of the given storage type
 int kinetic_pitch(int nnode, int f_dtype);
-// launch shape candidates (vectors per lane, lanes per row) for a row pitch; the first is the default
+// where the alpha / beta / w' tables of the linear rows hold node j: BF16 rows keep the low halves of their
+// eight-node vectors first, then the high halves (lds_halves in kinetic_row.cuh)
+inline size_t tab_pos(size_t j, size_t pitch, int f_dtype)
+{
+    return f_dtype == FDTD_DF_BF16 ? (j >> 2 & 1) * (pitch / 2) + (j >> 3) * 4 + (j & 3) : j;
+}
+// launch shape candidates (vectors per lane, lanes per row) for a row pitch, and the default one
 int kinetic_candidates(int pitch, int f_dtype, int (*out)[2]);
+void kinetic_default_shape(int pitch, int f_dtype, int *vpl, int *l);
 // returns cudaErrorInvalidValue for an unsupported combination; vpl <= 0 picks the default shape,
 // bps > 0 caps the CTAs per SM; stages > 0 (FP32 / BF16 storage) selects the bulk-copy ring kernel
 // with that many shared-memory stages (kinetic_ring.cu)

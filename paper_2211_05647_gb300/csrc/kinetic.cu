@@ -38,7 +38,45 @@ int kinetic_candidates(int nnode_pitch, int f_dtype, int (*out)[2])
     return kinetic_shape_candidates(nnode_pitch / vec, out);
 }
 
+// The default row shape (vectors per lane, lanes per row): it fixes the order J is summed in, so it follows the row
+// alone, never the number of rows (a sub-domain sums in the whole grid's order).  Timed inside whole steps on rows
+// of 15 MB to 1.5 GB of delta f: eight vectors a lane for FP32 rows of 64 and 128 (1.5 GB: 0.477 / 0.480 ms against
+// 0.502 / 0.500 with four), sixteen for rows of 256 (a little ahead at every size), two of eight for the 32-node rows
+// (0.489 against 0.553).  BF16 rows sum as four vectors a lane: another order of their FP32 sums moves J by a few
+// roundings, which the stochastic rounding of every node then turns into other codes.
+void kinetic_default_shape(int pitch, int f_dtype, int *vpl, int *l)
+{
+    int c[32][2];
+    kinetic_candidates(pitch, f_dtype, c);
+    const int V = pitch / (f_dtype == FDTD_DF_BF16 ? 8 : (f_dtype == FDTD_DF_F64 ? 2 : 4));
+    *vpl = c[0][0];
+    if (f_dtype == FDTD_DF_F32) {
+        if (V == 8) *vpl = 2;
+        else if (V == 64 || V == 128) *vpl = 8;
+        else if (V == 256) *vpl = 16;
+    }
+    *l = V / *vpl;
+}
+
+// How the default shape runs, by the bytes of delta f (same results either way).  Long FP32 rows beyond L2 go
+// through the bulk-copy ring (256 vectors, 3.4 GB: 1.01 against 1.07 ms; 128 and 64, 1.5 GB: 0.468 / 0.465 against
+// 0.480 / 0.477 at two CTAs a SM and 0.500 / 0.491 uncapped); the middle FP32 rows gain from fewer CTAs a SM (16
+// vectors: 0.471 at three against 0.510; 0.3 GB 98 against 104 us).  BF16 rows and the shortest FP32 ones lose with
+// either.
+void kinetic_default_run(int pitch, int f_dtype, int64_t nslots, int l, int *bps, int *stages)
+{
+    *bps = *stages = 0;
+    if (f_dtype != FDTD_DF_F32) return;
+    const int V = pitch / 4;
+    const int64_t bytes = nslots * pitch * 4;
+    if (V == 256 && bytes >= (int64_t)512 << 20) *stages = 3;
+    else if ((V == 64 || V == 128) && bytes >= (int64_t)256 << 20) *stages = 4;
+    if (*stages && !kinetic_ring_fits(pitch, f_dtype, l, *stages)) *stages = 0;
+    if (!*stages) *bps = V == 64 || V == 128 ? 2 : (V == 16 || V == 32 ? 3 : 0);
+}
+
 cudaError_t dispatch_kinetic_bf16(cudaStream_t st, const KinArgs<float> &a, int num_sms, int vpl, int l, int bps);
+cudaError_t dispatch_kinetic_bf16_wide(cudaStream_t st, const KinArgs<float> &a, int num_sms);
 cudaError_t dispatch_kinetic_f64(cudaStream_t st, const KinArgs<double> &a, int num_sms, int vpl, int l, int bps);
 
 template <>
@@ -47,10 +85,12 @@ cudaError_t launch_kinetic<float>(cudaStream_t st, const KinArgs<float> &a, int 
 {
     if (a.nslots == 0) return cudaSuccess;
     if (vpl <= 0) {
-        int c[8][2];
-        kinetic_candidates(a.pitch, f_dtype, c);
-        vpl = c[0][0];
-        l = c[0][1];
+        // BF16 rows of 16 to 128 vectors: eight a lane (1.5 GB, V = 64: 0.49 ms against 0.60 with four; V = 16: 0.51
+        // against 0.62), the four-vector shape's J
+        const int V = a.pitch / 8;
+        if (f_dtype == FDTD_DF_BF16 && V >= 16 && V <= 128) return dispatch_kinetic_bf16_wide(st, a, num_sms);
+        kinetic_default_shape(a.pitch, f_dtype, &vpl, &l);
+        kinetic_default_run(a.pitch, f_dtype, a.nslots, l, &bps, &stages);
     }
     if (stages > 0) return launch_kinetic_ring(st, a, f_dtype, num_sms, vpl, l, bps, stages);
     if (f_dtype == FDTD_DF_F32) return dispatch_kinetic<float, float>(st, a, num_sms, vpl, l, bps);
@@ -64,12 +104,7 @@ cudaError_t launch_kinetic<double>(cudaStream_t st, const KinArgs<double> &a, in
 {
     if (a.nslots == 0) return cudaSuccess;
     if (stages > 0) return cudaErrorInvalidValue;   // the ring kernel streams FP32 / BF16 rows only
-    if (vpl <= 0) {
-        int c[8][2];
-        kinetic_candidates(a.pitch, f_dtype, c);
-        vpl = c[0][0];
-        l = c[0][1];
-    }
+    if (vpl <= 0) kinetic_default_shape(a.pitch, f_dtype, &vpl, &l);
     if (f_dtype == FDTD_DF_F64) return dispatch_kinetic_f64(st, a, num_sms, vpl, l, bps);
     return cudaErrorInvalidValue;
 }

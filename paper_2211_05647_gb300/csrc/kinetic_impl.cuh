@@ -7,7 +7,7 @@
 
 namespace fp {
 
-template <typename TS, typename TA, int VPL, int L>
+template <typename TS, typename TA, int VPL, int L, int VS = VPL>   // VS: vectors a partial sum (row_update_to)
 __global__ void __launch_bounds__(256) k_kinetic(KinArgs<TA> a)
 {
     pdl_enter();
@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(256) k_kinetic(KinArgs<TA> a)
         const int64_t row_next = row + nw * R;
         cell_next = row_next < a.nslots ? __ldg(a.slot_cell + row_next) : 0;
         TA s = TA(0), c = TA(0);
-        if (valid) row_update<TS, TA, VPL, L>(rp, v, s_al, s_be, s_w, nE, l, (uint32_t)(row + a.slot_base), step, key, s, c);
+        if (valid) row_update<TS, TA, VPL, L, VS>(rp, v, s_al, s_be, s_w, nE, l, (uint32_t)(row + a.slot_base), step, key, s, c);
         const TA J = row_reduce<TA, L>(s, c);
         if (valid && l == 0) {
             if (a.store_j) a.jslot[row] = J;
@@ -56,10 +56,10 @@ __global__ void __launch_bounds__(256) k_kinetic(KinArgs<TA> a)
     }
 }
 
-template <typename TS, typename TA, int VPL, int L>
+template <typename TS, typename TA, int VPL, int L, int VS = VPL>
 cudaError_t run_kinetic(cudaStream_t st, const KinArgs<TA> &a, int num_sms, int blocks_per_sm)
 {
-    auto kern = k_kinetic<TS, TA, VPL, L>;
+    auto kern = k_kinetic<TS, TA, VPL, L, VS>;
     const size_t smem = 3 * (size_t)a.pitch * sizeof(TA);
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);

@@ -66,6 +66,15 @@ __device__ __forceinline__ void lds(const float *p, float *x)
         x[4 * q] = t.x; x[4 * q + 1] = t.y; x[4 * q + 2] = t.z; x[4 * q + 3] = t.w;
     }
 }
+// the eight table values of BF16 vector vi: nodes 0..3 of every vector, then nodes 4..7 (tab_pos), so that lanes
+// on consecutive vectors read consecutive 16-byte words.  Node order puts them 32 bytes apart: two-way bank
+// conflicts and half of all shared-memory wavefronts at eight lanes a row (1 KB rows of 512 nodes, 300 k of them:
+// 136 -> 104 us)
+__device__ __forceinline__ void lds_halves(const float *tab, int vi, int half, float *x)
+{
+    lds<4>(tab + 4 * vi, x);
+    lds<4>(tab + half + 4 * vi, x + 4);
+}
 template <int VEC>
 __device__ __forceinline__ void lds(const double *p, double *x)
 {
@@ -140,28 +149,35 @@ struct Store<__nv_bfloat16> {
 // terms, and which takes a fifth of the row's instructions.  BF16 rows run on
 // the two-lane FP32 instructions: node pairs (2t, 2t+1) get alpha df + (beta nE)
 // with the roundings of the scalar fma, and the sum is kept as two partial sums
-// (even and odd nodes) added at the end.
-template <typename TS, typename TA, int VPL, int L, typename Put>
+// (even and odd nodes) added at the end.  VS = VPL / 2 (BF16 rows): the lane
+// forms the sums of two lanes of the (VS, 2 L) shape, l and l + L, and adds them
+// as that shape's first reduction level does: J is the narrower shape's bit for
+// bit, with VPL loads in flight a lane.
+template <typename TS, typename TA, int VPL, int L, int VS, typename Put>
 __device__ __forceinline__ void row_update_to(const typename Vec<TS>::type *v, const TA *al_tab, const TA *be_tab,
                                               const TA *w_tab, TA nE, int l, uint32_t row_id, int64_t step, uint2 key,
                                               TA &s, TA &c, Put &&put)
 {
     constexpr int VEC = Vec<TS>::n;
     if constexpr (std::is_same<TS, __nv_bfloat16>::value) {
-        uint64_t s2 = f2(0.0f, 0.0f);
+        constexpr int NG = VPL / VS;
+        static_assert(NG == 1 || NG == 2, "one or two partial sums a lane");
+        uint64_t s2[NG];
+#pragma unroll
+        for (int g = 0; g < NG; ++g) s2[g] = f2(0.0f, 0.0f);
         const uint64_t ne2 = f2(nE, nE);
 #pragma unroll
         for (int q = 0; q < VPL; ++q) {
             const int vi = q * L + l;
             float x[VEC], al[VEC], be[VEC], w[VEC];
             unpack(v[q], x);
-            lds<VEC>(al_tab + vi * VEC, al);
-            lds<VEC>(be_tab + vi * VEC, be);
-            lds<VEC>(w_tab + vi * VEC, w);
+            lds_halves(al_tab, vi, VPL * L * 4, al);
+            lds_halves(be_tab, vi, VPL * L * 4, be);
+            lds_halves(w_tab, vi, VPL * L * 4, w);
 #pragma unroll
             for (int t = 0; t < VEC; t += 2) {
                 const uint64_t xn = f2_fma(f2(al[t], al[t + 1]), f2(x[t], x[t + 1]), f2_mul(f2(be[t], be[t + 1]), ne2));
-                s2 = f2_fma(f2(w[t], w[t + 1]), xn, s2);
+                s2[q % NG] = f2_fma(f2(w[t], w[t + 1]), xn, s2[q % NG]);
                 const float2 xs = f2_split(xn);
                 x[t] = xs.x;
                 x[t + 1] = xs.y;
@@ -169,9 +185,16 @@ __device__ __forceinline__ void row_update_to(const typename Vec<TS>::type *v, c
             const uint4 ctr = make_uint4(row_id, (uint32_t)vi, (uint32_t)step, (uint32_t)(step >> 32));
             put(vi, Store<TS>::pack(x, ctr, key));
         }
-        const float2 ss = f2_split(s2);
+        const float2 ss = f2_split(s2[0]);
         s = ss.x + ss.y;
         c = TA(0);
+        if constexpr (NG == 2) {
+            const float2 st = f2_split(s2[1]);
+            TA hi, lo;
+            two_sum(s, st.x + st.y, hi, lo);
+            s = hi;
+            c = lo;
+        }
     } else {
 #pragma unroll
         for (int q = 0; q < VPL; ++q) {
@@ -201,12 +224,12 @@ __device__ __forceinline__ void row_update_to(const typename Vec<TS>::type *v, c
 }
 
 // the same in place on a row in global memory (streaming stores)
-template <typename TS, typename TA, int VPL, int L>
+template <typename TS, typename TA, int VPL, int L, int VS = VPL>
 __device__ __forceinline__ void row_update(typename Vec<TS>::type *rp, const typename Vec<TS>::type *v,
                                            const TA *al_tab, const TA *be_tab, const TA *w_tab, TA nE, int l,
                                            uint32_t row_id, int64_t step, uint2 key, TA &s, TA &c)
 {
-    row_update_to<TS, TA, VPL, L>(v, al_tab, be_tab, w_tab, nE, l, row_id, step, key, s, c,
+    row_update_to<TS, TA, VPL, L, VS>(v, al_tab, be_tab, w_tab, nE, l, row_id, step, key, s, c,
                                   [&](int vi, const typename Vec<TS>::type &x) { __stcs(rp + vi, x); });
 }
 

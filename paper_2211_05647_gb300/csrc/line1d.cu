@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(kLineThreads, 1) k_line1d(LineArgs<TA> a)
                     for (int q = 0; q < VPL; ++q) v[q] = rp[q * L + l];
                     node = s_node[r];
                     const TA nE = s_dn[r] * sE[node];
-                    row_update_to<TS, TA, VPL, L>(v, s_al, s_be, s_w, nE, l, (uint32_t)(s0 + r), step, key, sm, cm,
+                    row_update_to<TS, TA, VPL, L, VPL>(v, s_al, s_be, s_w, nE, l, (uint32_t)(s0 + r), step, key, sm, cm,
                                                   [&](int vi, const V &x) { rp[vi] = x; });
                 }
                 const TA J = row_reduce<TA, L>(sm, cm);
@@ -256,23 +256,30 @@ cudaError_t run_line(cudaStream_t st, const LineArgs<TA> &a, int ctas)
     return cudaLaunchKernelEx(&cfg, kern, a);
 }
 
-// FP32 and BF16 rows take the shapes launch_kinetic picks by default (four vectors a lane), so J's sums are
-// formed in the same order.
+// FP32 and BF16 rows take the shape launch_kinetic picks by default, so J's sums are formed in the same order.
 template <typename TS, typename TA>
 cudaError_t dispatch_line(cudaStream_t st, const LineArgs<TA> &a, int ctas)
 {
-    switch (a.pitch / Vec<TS>::n) {
-    case 0:   // no plasma
-    case 1: return run_line<TS, TA, 1, 1>(st, a, ctas);
-    case 2: return run_line<TS, TA, 2, 1>(st, a, ctas);
-    case 4: return run_line<TS, TA, 4, 1>(st, a, ctas);
-    case 8: return run_line<TS, TA, 4, 2>(st, a, ctas);
-    case 16: return run_line<TS, TA, 4, 4>(st, a, ctas);
-    case 32: return run_line<TS, TA, 4, 8>(st, a, ctas);
-    case 64: return run_line<TS, TA, 4, 16>(st, a, ctas);
-    case 128: return run_line<TS, TA, 4, 32>(st, a, ctas);
-    default: return cudaErrorInvalidValue;
+    int vpl = 1, l = 1;   // no plasma
+    if (a.pitch) kinetic_default_shape(a.pitch, std::is_same<TS, float>::value ? FDTD_DF_F32 : FDTD_DF_BF16, &vpl, &l);
+    switch (vpl * 64 + l) {
+#define FP_LINE(VPL_, L_) \
+    case VPL_ * 64 + L_: return run_line<TS, TA, VPL_, L_>(st, a, ctas);
+    FP_LINE(1, 1) FP_LINE(2, 1) FP_LINE(4, 1) FP_LINE(4, 4) FP_LINE(4, 8)
+    default: break;
     }
+    if constexpr (std::is_same<TS, float>::value) {
+        switch (vpl * 64 + l) {
+            FP_LINE(2, 4) FP_LINE(8, 8) FP_LINE(8, 16)
+        default: return cudaErrorInvalidValue;
+        }
+    } else {
+        switch (vpl * 64 + l) {
+            FP_LINE(4, 2) FP_LINE(4, 16) FP_LINE(4, 32)
+        default: return cudaErrorInvalidValue;
+        }
+    }
+#undef FP_LINE
 }
 
 // FP64 rows: the shape with the fewest FP64 instructions on the busiest sub-core, each of which takes 64 cycles
