@@ -330,13 +330,41 @@ dim3 stencil_block(const fdtd_plasma *h)
     return h->g.ndim == 3 ? dim3(32, 4, 2) : dim3(32, 8, 1);
 }
 
-// cells per thread of the curl stencils: tuned, else 4 in 2-D (measured
-// faster on GB300) and 1 in 3-D (the four-cell 3-D kernels need 80 registers
-// and lose more to the lower occupancy than they save in instructions)
+// cells per thread of the curl stencils: tuned, else by size.  2-D: four from 1.5 M cells (2 M cells 16.9 against
+// 18.8 us a step, 4 M 23.6 against 35), one below, where the launch is short and a thread's four cells one after
+// the other make it longer (1 M 11.7 against 10.6, 512^2 8.7 against 4.9).  3-D: one (the four-cell 3-D kernels
+// need 80 registers and lose more to the lower occupancy than they save in instructions).
 int stencil_cpt(const fdtd_plasma *h)
 {
     if (h->st_cpt > 0) return h->st_cpt;
-    return h->g.ndim == 2 ? 4 : 1;
+    return h->g.ndim == 2 && h->nx * h->ny >= (int64_t)3 << 19 ? 4 : 1;
+}
+
+// Stencils of a handle that the tuning cache knows nothing about (FP32, nx a multiple of 4): from the sizes where
+// the fields no longer live in L2,
+//  2-D whole grids of 6 M cells and more: the fused E + H column march, 4 rows a segment, 8 from 32 M cells
+//      (us a step against the separate passes: 3000^2 51 / 59, 4096^2 80 / 107, 8192^2 263 / 384; 2048^2, in L2,
+//      27 / 24).  Its second field set must stay below a sixteenth of the device's memory.
+//  3-D grids of 12 M cells and more: the TMA columns, 12 planes a block (256^3 240 / 265, 512^3 1518 / 2019;
+//      192^3 129 / 118).
+// Results are the same bit for bit.
+void default_stencils(fdtd_plasma *h)
+{
+    if (h->st_bx > 0 || h->g.precision != FDTD_F32 || h->nx % 4) return;
+    const int64_t cells = h->nx * h->ny * h->nz;
+    if (h->g.ndim == 2 && !h->sd_on && cells >= 6000000) {
+        size_t avail = 0, total = 0;
+        if (cudaMemGetInfo(&avail, &total) != cudaSuccess) {
+            cudaGetLastError();
+            return;
+        }
+        if ((size_t)cells * 3 * 4 > total / 16) return;
+        h->auto_fuse_rows = cells >= 32000000 ? 8 : 4;
+        h->fuse_by_rule = 1;
+    } else if (h->g.ndim == 3 && cells >= 12000000) {
+        h->st_tz = 12;
+        h->st_bx = 32; h->st_by = 8; h->st_bz = 1; h->st_cpt = 1;
+    }
 }
 
 template <typename T>
@@ -686,6 +714,15 @@ bool fused_stencils(const fdtd_plasma *h)
 {
     const bool on = h->fuse || (h->auto_fuse_rows > 0 && h->g.ndim == 2);
     return on && h->g.ndim >= 2 && h->g.precision == FDTD_F32 && h->f2[FDTD_EZ] != nullptr;
+}
+
+// an explicit choice of the separate passes (a stencil option) ends the size rule's fused pass
+void end_fuse_rule(fdtd_plasma *h)
+{
+    if (!h->fuse_by_rule) return;
+    h->fuse_by_rule = 0;
+    h->auto_fuse_rows = 0;
+    if (!h->fuse) free_second_set(h);
 }
 
 // rows per segment of the 2-D column march: the option's when fusion was asked for, else the autotuner's
@@ -1046,7 +1083,10 @@ int create_impl(const fdtd_grid_desc *g, const fdtd_runtime_desc *rt, fdtd_plasm
     h->diag_out = (double *)dalloc(h, 8 * sizeof(double));
     if (!h->mur_state || !h->d_step || !h->d_src || !h->d_err || !h->diag_partials || !h->diag_out)
         return bail(FDTD_ERR_NOMEM, "small allocation failed");
-    if (g->ndim >= 2) apply_cached_stencil(h);
+    if (g->ndim >= 2) {
+        apply_cached_stencil(h);
+        default_stencils(h);
+    }
     rc = fdtd_plasma_reset(h);
     if (rc != FDTD_OK) {
         g_create_error = h->err;
@@ -1106,6 +1146,7 @@ int fdtd_plasma_set_option(fdtd_plasma_t h, int option, int64_t value)
         CK(h, cudaStreamSynchronize(h->stream));
         drop_graphs(h);
         h->fuse = (int)value;
+        if (!value) end_fuse_rule(h);
         if (!h->fuse && h->auto_fuse_rows <= 0) free_second_set(h);
         return FDTD_OK;
     }
@@ -1127,6 +1168,7 @@ int fdtd_plasma_set_option(fdtd_plasma_t h, int option, int64_t value)
         CK(h, cudaStreamSynchronize(h->stream));
         drop_graphs(h);
         h->st_tz = (int)value;
+        end_fuse_rule(h);
         if (value > 0) { h->st_bx = 32; h->st_by = 8; h->st_bz = 1; h->st_cpt = 1; }
         return FDTD_OK;
     }
@@ -1893,6 +1935,7 @@ int fdtd_plasma_autotune(fdtd_plasma_t h, fdtd_tune_result *out)
     h->steps_done = steps;
     dfree(h, blob);
     drop_graphs(h);
+    h->fuse_by_rule = 0;   // the tuner's choice now
     return rc != FDTD_OK ? rc : rc2;
 }
 

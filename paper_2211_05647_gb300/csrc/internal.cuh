@@ -416,6 +416,7 @@ struct fdtd_plasma {
     void *psi2[12];
     int fuse;                 // FDTD_OPT_FUSED_STENCILS (default 0)
     int fuse_rows;            // FDTD_OPT_FUSED_ROWS: 2-D column-march rows per block (0: the 64 x 16 tiles)
+    int fuse_by_rule;         // auto_fuse_rows comes from the size rule at create (an explicit stencil option ends it)
     int auto_fuse_rows;       // the autotuner's choice on 2-D FP32 grids: > 0 runs the fused column march
     // guard bytes around every device allocation ($FDTD_PLASMA_CANARIES=1 at create)
     int canary;
