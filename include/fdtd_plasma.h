@@ -416,10 +416,11 @@ int fdtd_plasma_set_recording(fdtd_plasma_t h, float *samples, int64_t capacity,
  *   forward  : y[b] = MLP(x[b]) for x [batch][17]
  *   loss_grad: loss = mean (y - target)^2 and its gradient (packed like the
  *              parameters, overwritten) -- forward and backward contractions
- *              on BF16 tensor-core tiles with FP32 accumulation, one CTA per
+ *              on BF16 tensor-core tiles with FP32 accumulation, four CTAs per
  *              128-row tile, the tiles' gradients summed in a fixed order
  *              (deterministic); workspace of fdtd_mlp_workspace_bytes(batch)
- *              bytes (one gradient per tile: about 74 KB per 128 rows)
+ *              bytes (a gradient and the rows of each 128-row tile, about 88 KB, and
+ *              the BF16 weights, 80 KB)
  *   adam     : one Adam step (Kingma & Ba, bias-corrected, step count t >= 1)
  *              on params with first / second moments m, v. */
 size_t fdtd_mlp_workspace_bytes(int64_t batch);
@@ -464,8 +465,8 @@ int fdtd_mlp_adam(float *params, const float *grad, float *m, float *v, int64_t 
  *   fdtd_mlp_gather would give, then the Adam step of fdtd_mlp_adam with step
  *   count iter0 + b + 1 and the cosine-decayed rate lr (1 + cos(pi (iter0 + b)
  *   / total_iters)) / 2 -- bit for bit those calls, in two kernel launches a
- *   batch (the rows are read through the permutation; the tiles' gradients
- *   are summed and applied in one kernel).  *loss_mean (device double)
+ *   batch (the tiles' gradients are summed and applied in one kernel, which
+ *   also takes the next batch's rows through the permutation).  *loss_mean (device double)
  *   receives the mean of the batch losses.  m, v: FDTD_MLP_NPARAMS floats
  *   each (zeroed by the caller before the first epoch); grad is not used (may
  *   be NULL); workspace of fdtd_mlp_train_workspace_bytes(batch) bytes.
