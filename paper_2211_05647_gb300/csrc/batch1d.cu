@@ -911,10 +911,10 @@ int fdtd_batch_read(fdtd_batch_t b, int32_t run, int which, void *dst, size_t by
         const size_t row = (size_t)b->nnode * b->df_esz, dp = (size_t)b->pitch * b->df_esz;
         e = copy_rows(b->stream, dst, (char *)b->df + b->row_off[run] * dp, b->nslot[run], row, dp, kind, true);
     } else {
-        const char *src = which == FDTD_EX   ? (char *)b->E + b->e_off[run] * b->esz
+        char *src = which == FDTD_EX   ? (char *)b->E + b->e_off[run] * b->esz
                           : which == FDTD_HY ? (char *)b->H + b->h_off[run] * b->esz
                                              : (char *)b->jslot + b->row_off[run] * b->esz;
-        e = cudaMemcpyAsync(dst, src, bytes, kind, b->stream);
+        e = copy_linear(b->stream, dst, src, bytes, kind, true);
     }
     if (e == cudaSuccess && !dst_is_device) e = cudaStreamSynchronize(b->stream);
     if (e != cudaSuccess) return bfail(b, FDTD_ERR_CUDA, "read: %s", cudaGetErrorString(e));

@@ -2007,8 +2007,7 @@ static int copy_quantity(fdtd_plasma_t h, int which, void *host_or_dev, size_t b
         CK(h, copy_rows(h->stream, host_or_dev, rows, h->nkin, row, dpitch, kind, out));
     } else {
         void *dev = which == FDTD_J ? h->jslot : h->f[which];
-        if (out) CK(h, cudaMemcpyAsync(host_or_dev, dev, bytes, kind, h->stream));
-        else CK(h, cudaMemcpyAsync(dev, host_or_dev, bytes, kind, h->stream));
+        CK(h, copy_linear(h->stream, host_or_dev, dev, bytes, kind, out));
     }
     if (!is_device) {
         int errw = 0;

@@ -284,6 +284,9 @@ cudaError_t launch_compact_scatter(cudaStream_t st, const double *d, const Compa
 // dst[i] = (float)src[i], i < n (round to nearest, as the host conversion)
 cudaError_t launch_to_f32(cudaStream_t st, const double *src, float *dst, int64_t n);
 
+// bytes between one of the solver's arrays and the caller's memory (out: to the caller), stream-ordered; kind says
+// where the caller's memory is (rows.cu)
+cudaError_t copy_linear(cudaStream_t st, void *theirs, void *ours, size_t bytes, cudaMemcpyKind kind, bool out);
 // delta-f rows between the padded layout (pitch bytes apart) and the packed one of read / write_fields; out:
 // padded -> packed.  kind says where the packed side is (rows.cu)
 cudaError_t copy_rows(cudaStream_t st, void *packed, void *padded, int64_t rows, size_t row, size_t pitch,

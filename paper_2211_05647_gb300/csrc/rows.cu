@@ -1,6 +1,11 @@
-// rows.cu -- delta-f rows between the solver's padded layout ([row][pitch]) and
-// the packed [row][nnode] layout of fdtd_plasma_read_fields / write_fields, both
-// in device memory.
+// rows.cu -- copies between the solver's arrays and a caller's device memory:
+// linear ones, and delta-f rows between the padded layout ([row][pitch]) and the
+// packed [row][nnode] layout of fdtd_plasma_read_fields / write_fields.
+//
+// A cudaMemcpyAsync inside device memory occupies the stream for about six
+// microseconds however small it is (reading E, H, J and delta f of 256 batched runs,
+// 1024 copies of 0.05 - 2 MB: 6.2 ms); those of 16 KB to 16 MB run as a kernel that
+// starts while the work before it finishes (3.1 ms).
 //
 // A strided cudaMemcpy2D of short rows runs far below the copy bandwidth (rows of
 // 124 bytes, 1.2 M of them: 141 us; 64-byte rows, 33.5 M: 3.2 ms), so rows that are not
@@ -9,6 +14,8 @@
 // multiple of, consecutive threads on consecutive units of the packed side, the
 // row of a unit by one multiplication (exact below 2^31).  Bound by HBM
 // (the same rows: 51 us, and 0.62 ms as a linear copy).
+#include <algorithm>
+
 #include "internal.cuh"
 
 namespace fp {
@@ -42,6 +49,41 @@ __global__ void __launch_bounds__(256) k_rows_copy(U *__restrict__ dst, const U 
 }
 
 template <typename U>
+__global__ void __launch_bounds__(256) k_copy(U *__restrict__ dst, const U *__restrict__ src, uint32_t n)
+{
+    pdl_enter();
+    const uint32_t stride = gridDim.x * 256u * kRowsUnroll;
+    for (uint32_t i0 = blockIdx.x * (256u * kRowsUnroll) + threadIdx.x; i0 < n; i0 += stride) {
+        U v[kRowsUnroll];
+#pragma unroll
+        for (int q = 0; q < kRowsUnroll; ++q)
+            if (i0 + 256u * q < n) v[q] = src[i0 + 256u * q];
+#pragma unroll
+        for (int q = 0; q < kRowsUnroll; ++q)
+            if (i0 + 256u * q < n) dst[i0 + 256u * q] = v[q];
+    }
+}
+
+template <typename U>
+cudaError_t run_copy(cudaStream_t st, void *dst, const void *src, size_t bytes)
+{
+    const uint32_t n = (uint32_t)(bytes / sizeof(U));
+    const uint32_t blocks = std::min<uint32_t>((n + 256 * kRowsUnroll - 1) / (256 * kRowsUnroll), 152 * 8);
+    return launch_pdl(k_copy<U>, dim3(blocks), dim3(256), 0, st, static_cast<U *>(dst), static_cast<const U *>(src), n);
+}
+
+// whether kernels of the current device may read and write the caller's memory (a copy engine reaches other places)
+bool on_this_device(const void *p)
+{
+    int dev = 0;
+    cudaPointerAttributes at{};
+    if (cudaGetDevice(&dev) == cudaSuccess && cudaPointerGetAttributes(&at, p) == cudaSuccess)
+        return at.type == cudaMemoryTypeDevice && at.device == dev;
+    cudaGetLastError();
+    return false;
+}
+
+template <typename U>
 cudaError_t run(cudaStream_t st, void *dst, const void *src, int64_t rows, size_t row, size_t pitch, bool pack)
 {
     const uint32_t per = (uint32_t)(row / sizeof(U)), n = (uint32_t)(rows * per);
@@ -59,30 +101,43 @@ cudaError_t run(cudaStream_t st, void *dst, const void *src, int64_t rows, size_
 
 }  // namespace
 
+cudaError_t copy_linear(cudaStream_t st, void *theirs, void *ours, size_t bytes, cudaMemcpyKind kind, bool out)
+{
+    void *dst = out ? theirs : ours;
+    const void *src = out ? ours : theirs;
+    // up to 16 MB the six microseconds are more than the kernel takes; beyond, both run at the copy bandwidth.  The
+    // smallest keep the plain copy: a call with the pointer's check and a launch is a microsecond longer on the
+    // host, which bounds a program that reads a few kilobytes after every step (39 against 43 us a step and four
+    // reads)
+    if (kind == cudaMemcpyDeviceToDevice && bytes > 16384 && bytes <= (size_t)16 << 20 && on_this_device(theirs)) {
+        size_t u = 16;
+        while (u > 2 && (((uintptr_t)dst | (uintptr_t)src | bytes) & (u - 1))) u >>= 1;
+        switch (u) {
+        case 16: return run_copy<uint4>(st, dst, src, bytes);
+        case 8: return run_copy<uint2>(st, dst, src, bytes);
+        case 4: return run_copy<uint32_t>(st, dst, src, bytes);
+        default:
+            if (!(((uintptr_t)dst | (uintptr_t)src | bytes) & 1)) return run_copy<uint16_t>(st, dst, src, bytes);
+        }
+    }
+    return cudaMemcpyAsync(dst, src, bytes, kind, st);
+}
+
 cudaError_t copy_rows(cudaStream_t st, void *packed, void *padded, int64_t rows, size_t row, size_t pitch,
                       cudaMemcpyKind kind, bool out)
 {
     void *dst = out ? packed : padded;
     const void *src = out ? padded : packed;
-    if (row == pitch) return cudaMemcpyAsync(dst, src, (size_t)rows * row, kind, st);
-    if (kind == cudaMemcpyDeviceToDevice && rows > 0) {
-        // the kernel needs the caller's memory on this device (a copy engine reaches other places too)
-        int dev = 0;
-        cudaPointerAttributes at{};
-        if (cudaGetDevice(&dev) == cudaSuccess && cudaPointerGetAttributes(&at, packed) == cudaSuccess &&
-            at.type == cudaMemoryTypeDevice && at.device == dev) {
-            size_t u = 16;
-            while (u > 1 && (row % u || pitch % u || (uintptr_t)packed % u)) u >>= 1;
-            if (u >= 2 && (uint64_t)rows * (row / u) < ((uint64_t)1 << 31)) {
-                switch (u) {
-                case 16: return run<uint4>(st, dst, src, rows, row, pitch, out);
-                case 8: return run<uint2>(st, dst, src, rows, row, pitch, out);
-                case 4: return run<uint32_t>(st, dst, src, rows, row, pitch, out);
-                default: return run<uint16_t>(st, dst, src, rows, row, pitch, out);
-                }
-            }
-        } else {
-            cudaGetLastError();
+    if (row == pitch) return copy_linear(st, packed, padded, (size_t)rows * row, kind, out);
+    size_t u = 16;
+    while (u > 1 && (row % u || pitch % u || (uintptr_t)packed % u)) u >>= 1;
+    if (kind == cudaMemcpyDeviceToDevice && rows > 0 && u >= 2 && (uint64_t)rows * (row / u) < ((uint64_t)1 << 31) &&
+        on_this_device(packed)) {
+        switch (u) {
+        case 16: return run<uint4>(st, dst, src, rows, row, pitch, out);
+        case 8: return run<uint2>(st, dst, src, rows, row, pitch, out);
+        case 4: return run<uint32_t>(st, dst, src, rows, row, pitch, out);
+        default: return run<uint16_t>(st, dst, src, rows, row, pitch, out);
         }
     }
     return out ? cudaMemcpy2DAsync(packed, row, padded, pitch, row, rows, kind, st)

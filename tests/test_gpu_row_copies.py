@@ -48,3 +48,21 @@ def test_device_rows_equal_host_rows(nv, nvp, dtype):
     assert torch.equal(s.read("df").cpu().view(-1), vals)
     s.step(2)                                                     # padding nodes are still 0: J stays finite
     assert s.diagnostics()["finite"]
+
+
+@pytest.mark.parametrize("nz", [4095, 4096, 4097, 50001, 5000000])
+@pytest.mark.parametrize("prec", ["f32", "f64"])
+def test_linear_copies(nz, prec):
+    """Fields of a line around the sizes where the copy kernel takes over (16 KB) and hands back (16 MB), to and from
+    addresses aligned to one element only."""
+    import torch
+    from paper_2211_05647_gb300 import Solver
+    td = torch.float32 if prec == "f32" else torch.float64
+    s = Solver(dict(ndim=1, nz=nz, dx=1e-3, courant=0.5, precision=prec))
+    v = torch.randn(nz + 2, generator=torch.Generator().manual_seed(nz), dtype=td).cuda()
+    for off in (0, 1):
+        s.write("ex", v[off:off + nz + 1])
+        assert np.array_equal(s.read("ex", device=False), v[off:off + nz + 1].cpu().numpy())
+        buf = torch.zeros(nz + 2, dtype=td, device="cuda")
+        assert s.lib.fdtd_plasma_read_fields(s.h, 0, ctypes.c_void_p(buf[off:].data_ptr()), s.quantity_bytes("ex"), 1) == 0
+        assert torch.equal(buf[off:off + nz + 1], v[off:off + nz + 1]) and float(buf[(1 - off) * (nz + 1)]) == 0.0
