@@ -415,7 +415,7 @@ def batch_config(workload: str, specs, steps: int, warmup: int, autotune: bool, 
                          "alg_bytes_per_launch": alg_step * chunk,
                          "launch_ms": per_launch_ms, "peak_source": src},
             "step_hbm_frac_algorithmic": alg_step / (ms / steps / 1e3) / 1e9 / peak,
-            "gpu_launches": 2 * (steps // chunk + (1 if rem else 0))}
+            "gpu_launches": 3 * (steps // chunk + (1 if rem else 0))}   # sources, steps, step counter
 
 
 def closure_config(steps: int, warmup: int, engine: str, autotune: bool, local: int) -> dict:
@@ -991,7 +991,7 @@ def batch_bench(args, specs, rank, world, local):
                          "alg_bytes_per_launch": alg_step * chunk,
                          "launch_ms": per_launch_ms,
                          "peak_source": "MEASURED_PEAKS.json hbm_gbs" if peaks else "fallback"},
-            "gpu_launches": 2 * (args.steps // chunk + (1 if rem else 0)),
+            "gpu_launches": 3 * (args.steps // chunk + (1 if rem else 0)),   # sources, steps, step counter
             "clocks": clk,
             "e2e": {"value": job_rate(cells * args.steps, world, te) / 1e9, "unit": UNIT,
                     "h2d_bytes_per_step": h2d / args.steps, "d2h_bytes_per_step": d2h / args.steps}}
