@@ -216,11 +216,11 @@ __device__ __forceinline__ void nl_store(T *p, const NlVec<T, C> &x)
 template <typename T, int C, int L>
 __global__ void __launch_bounds__(256, 2) k_kinetic_nl_walk(KinArgs<T> a, int npar, int nperp, T inv_dv, T qm, T dt)
 {
-    pdl_enter();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T *s_al = reinterpret_cast<T *>(smem_raw), *s_be = s_al + a.pitch, *s_w = s_be + a.pitch;
-    for (int t = threadIdx.x; t < 3 * a.pitch; t += blockDim.x) s_al[t] = a.tab[t];
+    for (int t = threadIdx.x; t < 3 * a.pitch; t += blockDim.x) s_al[t] = a.tab[t];   // constant: before the wait
     __syncthreads();
+    pdl_enter();
     using V = NlVec<T, C>;
     constexpr int U = kNlU, R = 32 / L;
     const int lane = threadIdx.x & 31, sub = lane / L, l = lane % L;
@@ -421,7 +421,6 @@ struct F0Tab {
 template <typename T, int L>
 __global__ void __launch_bounds__(256) k_kinetic_f0(KinArgs<T> a, F0Args<T> f)
 {
-    pdl_enter();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int P = a.pitch;
     T *s = reinterpret_cast<T *>(smem_raw);
@@ -431,6 +430,7 @@ __global__ void __launch_bounds__(256) k_kinetic_f0(KinArgs<T> a, F0Args<T> f)
     }
     for (int t = threadIdx.x; t < 8 * P; t += blockDim.x) s[2 * P + t] = f.tab[t];
     __syncthreads();
+    pdl_enter();   // the tables are constant
     const F0Tab<T> tb{s, s + P, s + 2 * P, s + 3 * P, s + 4 * P, s + 5 * P, s + 6 * P, s + 7 * P, s + 8 * P, s + 9 * P};
 
     using V = typename Vec<T>::type;
