@@ -1505,18 +1505,22 @@ int fdtd_plasma_step(fdtd_plasma_t h, int64_t nsteps)
     }
     if (!h->graphs_valid) {
         ensure_second_set(h);
-        int rc = capture(h, 1, &h->g1);
-        if (rc == FDTD_OK) rc = capture(h, kChunk, &h->gk);
-        if (rc != FDTD_OK) {
-            drop_graphs(h);
-            return rc;
-        }
         h->gk_steps = kChunk;
         h->graphs_valid = 1;
     }
     // the remainder (< 32 steps) as 16-, 8-, 4-, 2- and 1-step graphs: few launches, and the fused
     // stencil pass inside each of them; the ones this call needs are captured before anything runs
     const int64_t rem = nsteps % h->gk_steps;
+    if (nsteps >= h->gk_steps && !h->gk)
+        if (const int rc = capture(h, kChunk, &h->gk); rc != FDTD_OK) {
+            drop_graphs(h);
+            return rc;
+        }
+    if ((rem & 1) && !h->g1)
+        if (const int rc = capture(h, 1, &h->g1); rc != FDTD_OK) {
+            drop_graphs(h);
+            return rc;
+        }
     for (int b = 3; b >= 0; --b) {
         if (!((rem >> (b + 1)) & 1) || h->gpow[b]) continue;
         const int rc = capture(h, 2 << b, &h->gpow[b]);
