@@ -556,10 +556,11 @@ cudaError_t part_h(fdtd_plasma *h, cudaStream_t st, int kstep, const FieldSet<T>
 
 // the work between the H and E updates: E-history push, kinetic update (E -= dt/eps0 J), closure, recorder.
 // J^{n+1/2} per slot is stored on the last step of a sequence (what read_fields and checkpoints see between
-// step calls) and on every step while the recorder, which reads it, is on.
+// step calls) and on every step while the recorder, which reads it, is on.  after_stencil: no call can come
+// between the H update and this (in a split step the caller may write delta f there).
 template <typename T>
 cudaError_t part_mid(fdtd_plasma *h, cudaStream_t st, int kstep, const FieldSet<T> &fs, cudaEvent_t *ev,
-                     bool last = true)
+                     bool last = true, bool after_stencil = true)
 {
     T *E = fs.f[pol_comp(h)];
     const bool rec = h->has_recording && sizeof(T) == 4;
@@ -569,6 +570,7 @@ cudaError_t part_mid(fdtd_plasma *h, cudaStream_t st, int kstep, const FieldSet<
         KinArgs<T> a = kin_args<T>(h, kstep);
         a.E = E;
         a.store_j = last || rec;
+        a.after_stencil = after_stencil;
         cudaError_t e;
         if (h->pl.evolve_f0) {
             const double vth = std::sqrt(kQe * h->pl.te_ev / kMe);
@@ -1554,7 +1556,8 @@ int fdtd_plasma_step_half(fdtd_plasma_t h, int half)
         h->sd_half = 1;
         return FDTD_OK;
     }
-    e = dbl ? part_mid<double>(h, h->stream, 0, f64, nullptr) : part_mid<float>(h, h->stream, 0, f32, nullptr);
+    e = dbl ? part_mid<double>(h, h->stream, 0, f64, nullptr, true, false)
+            : part_mid<float>(h, h->stream, 0, f32, nullptr, true, false);
     if (e == cudaSuccess) e = dbl ? part_e<double>(h, h->stream, 0, f64) : part_e<float>(h, h->stream, 0, f32);
     if (e == cudaSuccess) e = dbl ? part_ports<double>(h, h->stream, 0, f64) : part_ports<float>(h, h->stream, 0, f32);
     if (e == cudaSuccess) {

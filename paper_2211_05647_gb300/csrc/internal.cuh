@@ -115,6 +115,8 @@ struct KinArgs {
     int store_j;               // k_kinetic: store J^{n+1/2} per slot (the last step of a sequence, or
                                // when something reads it every step); E is updated either way
     int *err;                  // set to 1 if a bounded wait of the bulk-copy ring kernel gave up
+    int after_stencil;         // k_kinetic: the launch before this one is a stencil of the same sequence (it may
+                               // then start, and read its first rows, while that stencil finishes)
 };
 
 // Isotropic-F0 evolution (speed grid): per-node tables, each `pitch` long,

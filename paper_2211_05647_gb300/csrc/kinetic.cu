@@ -11,8 +11,8 @@
 //
 // Layout: rows of `pitch` elements, [slot][node], pitch = a power-of-two
 // number of 16-byte vectors >= nnode (padding nodes have alpha = beta = w = 0
-// and stay 0).  L lanes share a row, each lane holding VPL >= 4 vectors when
-// the row has that many; a warp covers 32/L rows.  The whole row is loaded
+// and stay 0).  L lanes share a row, each lane holding VPL vectors (two to
+// sixteen: kinetic_default_shape); a warp covers 32/L rows.  The whole row is loaded
 // before any arithmetic so each lane has VPL 16-byte loads in flight, the
 // loads/stores use the streaming (evict-first) cache hint because delta f is
 // far larger than L2, and the per-node tables sit in shared memory.

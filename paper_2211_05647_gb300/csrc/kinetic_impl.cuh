@@ -11,10 +11,11 @@ template <typename TS, typename TA, int VPL, int L, int VS = VPL>   // VS: vecto
 __global__ void __launch_bounds__(256) k_kinetic(KinArgs<TA> a)
 {
     // What no kernel before this one writes is fetched before the grid dependency: the tables, and of the first
-    // row group the cell index and the delta-f vectors.  Only this kernel writes delta f, and between two of its
-    // launches lies a stencil launch that waits for the first one before it lets the next start, so the rows are
-    // final; the loads then overlap the stencil's last wave (5 k rows of 1024 nodes on a 192 x 160 grid: 14.6 ->
-    // 12.3 us a step).
+    // row group the cell index and the delta-f vectors.  Within a sequence of steps only this kernel writes delta f,
+    // and between two of its launches lies a stencil launch that waits for the first one before it lets the next
+    // start, so the rows are final; the loads then overlap the stencil's last wave (5 k rows of 1024 nodes on a
+    // 192 x 160 grid: 14.6 -> 12.3 us a step).  The second half of a split step may follow a write of delta f
+    // instead, so it is launched without the overlap (a.after_stencil).
     extern __shared__ __align__(16) unsigned char smem_raw[];
     TA *s_tab = reinterpret_cast<TA *>(smem_raw);
     for (int t = threadIdx.x; t < 3 * a.pitch; t += blockDim.x) s_tab[t] = a.tab[t];
@@ -91,12 +92,13 @@ cudaError_t run_kinetic(cudaStream_t st, const KinArgs<TA> &a, int num_sms, int 
     const int64_t cap = (int64_t)num_sms * per_sm;
     if (blocks > cap) blocks = cap;
     if (blocks < 1) blocks = 1;
-    launch_pdl(kern, dim3((unsigned)blocks), dim3(256), smem, st, a);
+    if (a.after_stencil) launch_pdl(kern, dim3((unsigned)blocks), dim3(256), smem, st, a);
+    else launch_plain(kern, dim3((unsigned)blocks), dim3(256), smem, st, a);
     return cudaGetLastError();
 }
 
-// Shape candidates (VPL, L) for V vectors per row; the first is the default
-// (every lane keeps >= 4 sixteen-byte loads in flight when the row allows it).
+// Shape candidates (VPL, L) for V vectors per row.  The first keeps >= 4 sixteen-byte loads a lane in flight when the
+// row allows it; kinetic_default_shape takes it except where another measured faster.
 inline int kinetic_shape_candidates(int V, int (*out)[2])
 {
     static const int tab[][2] = {{1, 1},
