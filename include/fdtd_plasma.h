@@ -182,8 +182,13 @@ int fdtd_plasma_set_source(fdtd_plasma_t h, const fdtd_source_desc *src);
 int fdtd_plasma_set_plasma(fdtd_plasma_t h, const fdtd_plasma_desc *pl);
 
 /* Advance nsteps >= 0 steps, asynchronously on the handle's stream.  The
- * first call after a configuration change captures the step sequence into
- * CUDA graphs; later calls replay them. */
+ * step sequence runs as CUDA graphs of 32, 16, 8, 4, 2 and 1 steps, each
+ * captured when a call first needs it after a configuration change.  A 1-D
+ * grid whose state fits in the SMs' shared memory (linear delta f rows or no
+ * plasma; no ports, recorder or closure) takes any number of steps in one
+ * cooperative launch instead (FDTD_ERR_CUDA while the handle's stream is
+ * capturing, as the graphs' capture is); its bounded waits set the error word
+ * described at fdtd_selftest_wait_timeout. */
 int fdtd_plasma_step(fdtd_plasma_t h, int64_t nsteps);
 
 /* Advance nsteps >= 1 steps like fdtd_plasma_step, but launch each kernel
@@ -237,8 +242,9 @@ int fdtd_plasma_autotune(fdtd_plasma_t h, fdtd_tune_result *out);
 int fdtd_plasma_check_canaries(fdtd_plasma_t h, int64_t *corrupted);
 
 /* Self-test of the bounded waits (no counterpart in the paper): the tcgen05
- * kernels wait for their tensor-core results, and the TMA column stencils for
- * their plane loads, on mbarriers with an iteration or wall-clock limit, after which they
+ * kernels wait for their tensor-core results, the TMA column stencils for
+ * their plane loads, the bulk-copy ring for its chunks and the 1-D stepping kernel
+ * for its neighbours' edges with an iteration or wall-clock limit, after which they
  * set an error word (reported as FDTD_ERR_TIMEOUT by fdtd_plasma_diagnostics
  * and by host reads of fdtd_plasma_read_fields) and return instead of hanging.  This launches one
  * CTA that waits, with the same helper, on a barrier nothing arrives at, for
@@ -253,18 +259,26 @@ int fdtd_selftest_wait_timeout(uint32_t max_iter, int32_t *gave_up);
  * Synchronous, on the legacy stream; FDTD_ERR_INVAL for a bad argument. */
 int fdtd_selftest_timed_wait(uint32_t limit_us, int32_t *gave_up);
 
-/* Runtime options.  FDTD_OPT_FUSED_STENCILS (default 0): 1 makes the step
+/* Runtime options.  Without any, and without autotuned or cached shapes, the
+ * sizes choose: 2-D FP32 whole grids of 6 M cells and more (nx a multiple of
+ * 4) run the fused column march below when its second field set fits in a
+ * sixteenth of the device's memory, 3-D FP32 grids of 12 M cells and more the TMA
+ * columns of 12 planes, others the grid-of-cells kernels; setting
+ * FDTD_OPT_FUSED_STENCILS to 0 or FDTD_OPT_STENCIL_TZ ends the 2-D rule.
+ * Results are the same bit for bit.
+ * FDTD_OPT_FUSED_STENCILS (default 0): 1 makes the step
  * sequence on 2-D and 3-D FP32 grids fuse each E update with the next H update into
  * one pass (fields and CPML psi double-buffered: one extra copy of them is
  * allocated on first use; the fields are back in place when
  * fdtd_plasma_step returns).  It moves a third fewer bytes; in 3-D it is
  * slower than the two separate passes on GB300, in 2-D (the column march
- * below) faster on large grids, where fdtd_plasma_autotune selects it by
- * itself (fdtd_tune_result.fused_rows; half steps stay allowed then).
+ * below) faster on large grids, where the size rule or fdtd_plasma_autotune selects it
+ * (fdtd_tune_result.fused_rows; half steps stay allowed then).
  * Results equal the unfused sequence bit for bit in 2-D and where the 3-D TMA
  * column stencils below are selected (their fused pass then runs on
  * TMA-staged planes too), else up to FP32 rounding order.  0 turns the
- * option off (and frees the copy unless the autotuner chose the fused pass).
+ * option off (and frees the copy unless the autotuner chose the fused pass
+ * since).
  * FDTD_OPT_STENCIL_TZ: 0 selects the grid-of-cells stencil kernels; a value
  * tz in 1..1024 selects the TMA kernels (2-D and 3-D FP32, nx a multiple of 4):
  * 32 x 8 threads per block; in 3-D each block walks tz planes along z, in 2-D
@@ -278,7 +292,8 @@ int fdtd_selftest_timed_wait(uint32_t limit_us, int32_t *gave_up);
  * length's candidates (the ones fdtd_plasma_autotune times), stages 0 (the
  * register kernel) or 2..64 (the bulk-copy ring kernel: FP32 / BF16 rows of
  * the linear update, stages that fit in one CTA's shared memory); 0 returns
- * to the built-in default.
+ * to the built-in default, which follows the row's length and the bytes of
+ * delta f.  The order J is summed in follows (vpl, l).
  * Needs a plasma (after set_plasma).  The autotuner overwrites it.
  * FDTD_OPT_FUSED_ROWS (2-D fused pass, nx a multiple of 4): rows per block
  * segment of the column-march kernel (1..4096, default 8; each warp owns a

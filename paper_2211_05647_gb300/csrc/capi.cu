@@ -28,7 +28,7 @@ using namespace fp;
 
 namespace {
 
-constexpr int kChunk = 32;            // steps per replay of the chunk graph
+constexpr int kChunk = kSourceSteps;  // steps per replay of the chunk graph (the source's table holds as many)
 constexpr int kFuseRowsDefault = 8;   // rows per block segment of the 2-D fused column march
 constexpr uint64_t kStateMagic = 0x4644544450534d31ull;
 
@@ -312,7 +312,8 @@ Cpml<T> cpml_view(fdtd_plasma *h)
     return c;
 }
 
-Source source_view(fdtd_plasma *h)
+// the source as a step's kernels see it (kstep: the step's offset in its sequence)
+Source source_view(fdtd_plasma *h, int kstep = 0)
 {
     Source s{};
     if (!h->has_source) return s;
@@ -320,7 +321,7 @@ Source source_view(fdtd_plasma *h)
     s.amp = h->src.amp; s.fc = h->src.fc; s.tau = h->src.tau; s.t0 = h->src.t0; s.dt = h->dt;
     s.i = h->src.i; s.j = h->src.j; s.k = h->src.k;
     s.i0 = h->src.i0; s.i1 = h->src.i1; s.j0 = h->src.j0; s.j1 = h->src.j1;
-    s.val = h->d_src;
+    s.val = h->d_src + kstep;
     return s;
 }
 
@@ -526,7 +527,7 @@ cudaError_t part_h(fdtd_plasma *h, cudaStream_t st, int kstep, const FieldSet<T>
     const double mu0 = 1.0 / (kEps0 * kC0 * kC0);
     const T ch = (T)(h->dt / (mu0 * h->g.dx)), cph = (T)(h->dt / mu0);
     T *const *f = fs.f;
-    const Source src = source_view(h);
+    const Source src = source_view(h, kstep);
     if (h->g.ndim == 1)
         launch_h1d<T>(st, f[FDTD_EX], f[FDTD_HY], h->g.mur ? (T *)h->mur_state : nullptr, h->nz, ch, src, h->d_step,
                       kstep);
@@ -633,7 +634,7 @@ cudaError_t part_e(fdtd_plasma *h, cudaStream_t st, int kstep, const FieldSet<T>
 {
     const T ce = (T)(h->dt / (kEps0 * h->g.dx)), cpe = (T)(h->dt / kEps0);
     T *const *f = fs.f;
-    const Source src = source_view(h);
+    const Source src = source_view(h, kstep);
     if (h->g.ndim == 1) {
         const T m = (T)((kC0 * h->dt - h->g.dx) / (kC0 * h->dt + h->g.dx));
         launch_e1d<T>(st, f[FDTD_EX], f[FDTD_HY], h->nz, ce, src, h->d_step, kstep,
@@ -763,13 +764,13 @@ cudaError_t enqueue_seq(fdtd_plasma *h, cudaStream_t st, int nsteps)
                 const float ch = (float)(h->dt / (mu0 * h->g.dx)), cph = (float)(h->dt / mu0);
                 if (h->g.ndim == 3) {
                     if (!(tma_fused && launch_eh3d_tma(st, h->tma, fs.f, to.f, to.cp.psi, ce, cpe, ch, cph, fs.cp,
-                                                       source_view(h), h->d_step, k, h->st_tz, h->d_err)))
+                                                       source_view(h, k), h->st_tz, h->d_err)))
                         launch_eh3d(st, fs.f, to.f, to.cp.psi, h->nx, h->ny, h->nz, ce, cpe, ch, cph, fs.cp,
-                                    source_view(h), h->d_step, k);
+                                    source_view(h, k));
                 }
                 else
-                    launch_eh2d(st, fs.f, to.f, to.cp.psi, h->nx, h->ny, ce, cpe, ch, cph, fs.cp, source_view(h),
-                                h->d_step, k, fuse_rows_of(h));
+                    launch_eh2d(st, fs.f, to.f, to.cp.psi, h->nx, h->ny, ce, cpe, ch, cph, fs.cp, source_view(h, k),
+                                fuse_rows_of(h));
             }
             set ^= 1;
             e = part_ports<T>(h, st, k, to);
@@ -1078,7 +1079,7 @@ int create_impl(const fdtd_grid_desc *g, const fdtd_runtime_desc *rt, fdtd_plasm
     }
     h->mur_state = dalloc(h, 4 * 8);
     h->d_step = (int64_t *)dalloc(h, 256);
-    h->d_src = (double *)dalloc(h, 256);
+    h->d_src = (double *)dalloc(h, kSourceSteps * sizeof(double));
     h->d_err = (int *)dalloc(h, 256);
     h->diag_blocks = h->num_sms * 4;
     h->diag_partials = (double *)dalloc(h, (size_t)h->diag_blocks * 7 * sizeof(double));
@@ -1746,7 +1747,7 @@ int autotune_t(fdtd_plasma *h, fdtd_tune_result *out)
     T *f[6];
     for (int q = 0; q < 6; ++q) f[q] = reinterpret_cast<T *>(h->f[q]);
     const Cpml<T> cp = cpml_view<T>(h);
-    const Source src = source_view(h);
+    const Source src = source_view(h);   // (H updates at step offset 1: as most do, without the source's table)
     cudaStream_t st = h->stream;
     cudaEvent_t e0, e1;
     CK(h, cudaEventCreate(&e0));
@@ -1778,11 +1779,11 @@ int autotune_t(fdtd_plasma *h, fdtd_tune_result *out)
                 const double ms = time_ms([&] {
                     if (h->g.ndim == 2) {
                         launch_h2d<T>(st, f[FDTD_EZ], f[FDTD_HX], f[FDTD_HY], h->nx, h->ny, ch, cph, cp, src, h->d_step,
-                                      0, b, cpt);
+                                      1, b, cpt);
                         launch_e2d<T>(st, f[FDTD_EZ], f[FDTD_HX], f[FDTD_HY], h->nx, h->ny, ce, cpe, cp, src, h->d_step,
                                       0, b, cpt);
                     } else {
-                        launch_h3d<T>(st, f, h->nx, h->ny, h->nz, ch, cph, cp, src, h->d_step, 0, b, cpt);
+                        launch_h3d<T>(st, f, h->nx, h->ny, h->nz, ch, cph, cp, src, h->d_step, 1, b, cpt);
                         launch_e3d<T>(st, f, h->nx, h->ny, h->nz, ce, cpe, cp, src, h->d_step, 0, b, cpt);
                     }
                 });
@@ -1799,7 +1800,7 @@ int autotune_t(fdtd_plasma *h, fdtd_tune_result *out)
                 for (int rows : {32, 48, 64, 96, 128}) {
                     if (rows > 4 * h->ny) continue;
                     const double ms = time_ms([&] {
-                        launch_h2d_tma(st, h->tma, f, h->nx, h->ny, ch, cph, cp, src, h->d_step, 0, rows, h->d_err);
+                        launch_h2d_tma(st, h->tma, f, h->nx, h->ny, ch, cph, cp, src, h->d_step, 1, rows, h->d_err);
                         launch_e2d_tma(st, h->tma, f, h->nx, h->ny, ce, cpe, cp, src, rows, h->d_err);
                     });
                     if (ms < best * kTuneMargin) {
@@ -1813,7 +1814,7 @@ int autotune_t(fdtd_plasma *h, fdtd_tune_result *out)
                 for (int tz : {8, 12, 16, 24, 32}) {
                     if (tz > 2 * h->nz) continue;
                     const double ms = time_ms([&] {
-                        launch_h3d_tma(st, h->tma, f, h->nx, h->ny, h->nz, ch, cph, cp, src, h->d_step, 0, tz,
+                        launch_h3d_tma(st, h->tma, f, h->nx, h->ny, h->nz, ch, cph, cp, src, h->d_step, 1, tz,
                                        h->d_err);
                         launch_e3d_tma(st, h->tma, f, h->nx, h->ny, h->nz, ce, cpe, cp, src, tz, h->d_err);
                     });
@@ -1838,7 +1839,7 @@ int autotune_t(fdtd_plasma *h, fdtd_tune_result *out)
                     for (int q = 0; q < 12; ++q) po[q] = reinterpret_cast<float *>(h->psi2[q]);
                     for (int rows : {4, 8, 16, 32}) {
                         const double ms = time_ms([&] {
-                            launch_eh2d(st, f, fo, po, h->nx, h->ny, ce, cpe, ch, cph, cp, src, h->d_step, 0, rows);
+                            launch_eh2d(st, f, fo, po, h->nx, h->ny, ce, cpe, ch, cph, cp, src, rows);
                         });
                         if (ms < best * kTuneMargin) {
                             best = ms;

@@ -21,12 +21,13 @@ namespace fp {
 // ------------------------------------------------------------------- 1-D
 
 template <typename T>
-__global__ void k_h1d(const T *__restrict__ ex, T *__restrict__ hy, T *__restrict__ mur, int64_t nz, T ch, Source src,
-                      const int64_t *__restrict__ d_step, int kstep)
+__global__ void __launch_bounds__(256, 8) k_h1d(const T *__restrict__ ex, T *__restrict__ hy, T *__restrict__ mur,
+                                                int64_t nz, T ch, Source src, const int64_t *__restrict__ d_step,
+                                                int kstep)
 {
     pdl_enter();
     int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (k == 0) write_source(src, d_step, kstep);
+    write_source_block0(src, d_step, kstep);
     if (k < nz) hy[k] -= ch * (ex[k + 1] - ex[k]);   // mu0 dHy/dt = -dEx/dz
     if (mur) {                                       // E_1^n and E_{nz-1}^n for the Mur ends
         if (k == 1) mur[0] = ex[1];
@@ -58,14 +59,14 @@ __global__ void k_e1d(T *__restrict__ ex, const T *__restrict__ hy, int64_t nz, 
 // (2-D CPML cell updates h2d_pml / e2d_pml: stencil_common.cuh)
 
 template <typename T>
-__global__ void __launch_bounds__(256) k_h2d(const T *__restrict__ ez, T *__restrict__ hx, T *__restrict__ hy,
-                                             int64_t nx, int64_t ny, T ch, T cph, Cpml<T> cp, Source src,
-                                             const int64_t *__restrict__ d_step, int kstep)
+__global__ void __launch_bounds__(256, 8) k_h2d(const T *__restrict__ ez, T *__restrict__ hx, T *__restrict__ hy,
+                                                int64_t nx, int64_t ny, T ch, T cph, Cpml<T> cp, Source src,
+                                                const int64_t *__restrict__ d_step, int kstep)
 {
     pdl_enter();
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t j = (int64_t)blockIdx.y * blockDim.y + threadIdx.y;
-    if (i == 0 && j == 0) write_source(src, d_step, kstep);
+    write_source_block0(src, d_step, kstep);
     if (i >= nx || j >= ny) return;
     const int64_t c = j * nx + i;
     const T e = ez[c];
@@ -118,7 +119,7 @@ __global__ void __launch_bounds__(256) k_h3d(const T *__restrict__ ex, const T *
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t j = (int64_t)blockIdx.y * blockDim.y + threadIdx.y;
     const int64_t k = (int64_t)blockIdx.z * blockDim.z + threadIdx.z;
-    if (i == 0 && j == 0 && k == 0) write_source(src, d_step, kstep);
+    write_source_block0(src, d_step, kstep);
     if (i >= nx || j >= ny || k >= nz) return;
     const int64_t sxy = nx * ny;
     const int64_t c = k * sxy + j * nx + i;
@@ -221,7 +222,7 @@ __global__ void __launch_bounds__(256) k_h2d_v4(const float *__restrict__ ez, fl
     pdl_enter();
     const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t j = (int64_t)blockIdx.y * blockDim.y + threadIdx.y;
-    if (q == 0 && j == 0) write_source(src, d_step, kstep);
+    write_source_block0(src, d_step, kstep);
     const int64_t i0 = 4 * q;
     const bool live = i0 < nx && j < ny;
     const int64_t c = live ? j * nx + i0 : 0;
@@ -302,7 +303,7 @@ __global__ void __launch_bounds__(256) k_h3d_v4(const float *__restrict__ ex, co
     const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const int64_t j = (int64_t)blockIdx.y * blockDim.y + threadIdx.y;
     const int64_t k = (int64_t)blockIdx.z * blockDim.z + threadIdx.z;
-    if (q == 0 && j == 0 && k == 0) write_source(src, d_step, kstep);
+    write_source_block0(src, d_step, kstep);
     const int64_t i0 = 4 * q, sxy = nx * ny;
     const bool live = i0 < nx && j < ny && k < nz;
     const int64_t c = live ? k * sxy + j * nx + i0 : 0;
@@ -536,8 +537,7 @@ struct PsiOut {
 
 __global__ void __launch_bounds__(kEhX * kEhY, 3) k_eh3d(FieldPtrs in, FieldOut out, int64_t nx, int64_t ny, int64_t nz,
                                                      int tz, float ce, float cpe, float ch, float cph, Cpml<float> cin,
-                                                     PsiOut pout, Source src, const int64_t *__restrict__ d_step,
-                                                     int kstep)
+                                                     PsiOut pout, Source src)
 {
     pdl_enter();
     __shared__ float sH[2][3][kEhY + 2][kEhX + 2];   // H^{n+1/2}: x0-1..x0+32, y0-1..y0+8
@@ -547,12 +547,7 @@ __global__ void __launch_bounds__(kEhX * kEhY, 3) k_eh3d(FieldPtrs in, FieldOut 
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * kEhX + tx;
     const int64_t x0 = (int64_t)blockIdx.x * kEhX, y0 = (int64_t)blockIdx.y * kEhY, z0 = (int64_t)blockIdx.z * tz;
     const int64_t z1 = min(z0 + (int64_t)tz, nz);
-    const int64_t n1 = *d_step + kstep + 1;   // E^{n+1} is at t^{n+1}
-    if (tid == 0) {
-        s_g = src.kind && src.k >= z0 && src.k <= z1 ? (float)source_value(src, (double)n1 * src.dt) : 0.f;
-        if (src.kind && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0)
-            *src.val = source_value(src, (double)(n1 + 1) * src.dt);
-    }
+    if (tid == 0) s_g = src.kind ? (float)*src.val : 0.f;
     const int64_t sxy = nx * ny;
     // Staging of one plane: each thread fetches its share of the plane's H (with the -x / -y halo) and E'
     // (with the +x / +y halo) into registers, and later commits them to shared memory, so the global loads
@@ -717,7 +712,7 @@ __global__ void __launch_bounds__(kF2T) k_eh2d(const float *__restrict__ ez_in, 
                                                const float *__restrict__ hy_in, float *__restrict__ ez_out,
                                                float *__restrict__ hx_out, float *__restrict__ hy_out, int64_t nx,
                                                int64_t ny, float ce, float cpe, float ch, float cph, Cpml<float> cin,
-                                               PsiOut pout, Source src, const int64_t *__restrict__ d_step, int kstep)
+                                               PsiOut pout, Source src)
 {
     pdl_enter();
     __shared__ float sHx[kF2Y + 2][kF2X + 2], sHy[kF2Y + 2][kF2X + 2];   // x0-1..x0+64, y0-1..y0+16
@@ -726,12 +721,7 @@ __global__ void __launch_bounds__(kF2T) k_eh2d(const float *__restrict__ ez_in, 
     __shared__ float s_g;
     const int tid = threadIdx.x;
     const int64_t x0 = (int64_t)blockIdx.x * kF2X, y0 = (int64_t)blockIdx.y * kF2Y;
-    const int64_t n1 = *d_step + kstep + 1;
-    if (tid == 0) {
-        const bool near = src.kind && src.i >= x0 && src.i <= x0 + kF2X && src.j >= y0 && src.j <= y0 + kF2Y;
-        s_g = near ? (float)source_value(src, (double)n1 * src.dt) : 0.f;
-        if (src.kind && blockIdx.x == 0 && blockIdx.y == 0) *src.val = source_value(src, (double)(n1 + 1) * src.dt);
-    }
+    if (tid == 0) s_g = src.kind ? (float)*src.val : 0.f;
     for (int r = tid; r < (kF2Y + 2) * (kF2X + 2); r += kF2T) {
         const int rx = r % (kF2X + 2), ry = r / (kF2X + 2);
         const int64_t i = x0 - 1 + rx, j = y0 - 1 + ry;
@@ -808,25 +798,11 @@ __global__ void __launch_bounds__(kF2T) k_eh2d(const float *__restrict__ ez_in, 
 constexpr int kEh2W = 1;   // warps (128-column strips) per block: a block's slot frees as soon as its strip ends
 constexpr int kEh2D = 4;   // rows in each lane's copy ring
 
-// g(t^{n1}) in FP32, as the separate E kernel reads it; out of line because
-// only the thread at the source node calls it
-__device__ __noinline__ float source_f32(int kind, double amp, double fc, double tau, double t0, double dt, int64_t n1)
-{
-    Source s{};
-    s.kind = kind;
-    s.amp = amp;
-    s.fc = fc;
-    s.tau = tau;
-    s.t0 = t0;
-    s.dt = dt;
-    return (float)source_value(s, (double)n1 * dt);
-}
-
 __global__ void __launch_bounds__(32 * kEh2W, 22)
     k_eh2d_v4(const float *__restrict__ ez_in, const float *__restrict__ hx_in, const float *__restrict__ hy_in,
               float *__restrict__ ez_out, float *__restrict__ hx_out, float *__restrict__ hy_out, int64_t nx,
               int64_t ny, int rows, int ktop, float ce, float cpe, float ch, float cph, Cpml<float> cin, PsiOut pout,
-              Source src, const int64_t *__restrict__ d_step, int kstep)
+              Source src)
 {
     pdl_enter();
     const int lane = (int)(threadIdx.x & 31u), w = (int)(threadIdx.x >> 5);
@@ -840,9 +816,6 @@ __global__ void __launch_bounds__(32 * kEh2W, 22)
     const int j0 = seg * rows;
     const int j1 = j0 + rows < nyi ? j0 + rows : nyi;   // owned rows [j0, j1)
     const int jl = j1 < nyi ? j1 : nyi - 1;             // last row whose E^{n+1} is formed
-    const int64_t n1 = *d_step + kstep + 1;
-    if (src.kind && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0)
-        *src.val = source_value(src, (double)(n1 + 1) * src.dt);   // g(t^{n+2}) for a following unfused E
     if (xs >= nx) return;   // the whole warp is past the grid
     const bool live = i0 < nx;
     const int64_t xr = xs + 128;   // the column beyond the strip (lane 31's quad + 4)
@@ -960,7 +933,7 @@ __global__ void __launch_bounds__(32 * kEh2W, 22)
                     en.v[e] = rn_add(en.v[e], pml ? e2d_pml_io<float>(cin, pout.psi, own, nx, ny, i, j, ce, cpe, dHx, dHy)
                                                   : e2d_term(ce, dHx, dHy));
                     if (srow && e == src_e)
-                        en.v[e] = rn_add(en.v[e], source_f32(src.kind, src.amp, src.fc, src.tau, src.t0, src.dt, n1));
+                        en.v[e] = rn_add(en.v[e], (float)*src.val);
                 } else if (pml && own) {
                     e2d_psi_carry<float>(cin, pout.psi, nx, ny, i, j);
                 }
@@ -977,7 +950,7 @@ __global__ void __launch_bounds__(32 * kEh2W, 22)
                                                                          dHx, dHy)
                                                      : e2d_term(ce, dHx, dHy));
                 if (srow && src_r)
-                    enr = rn_add(enr, source_f32(src.kind, src.amp, src.fc, src.tau, src.t0, src.dt, n1));
+                    enr = rn_add(enr, (float)*src.val);
             }
         }
         float er = __shfl_down_sync(full, en.v[0], 1);
@@ -1042,8 +1015,7 @@ __global__ void k_advance(int64_t *d_step, int64_t by)
 static inline unsigned cdiv(int64_t a, int64_t b) { return (unsigned)((a + b - 1) / b); }
 
 void launch_eh2d(cudaStream_t st, float *const fin[6], float *const fout[6], float *const psi_out[12], int64_t nx,
-                 int64_t ny, float ce, float cpe, float ch, float cph, Cpml<float> cin, Source src,
-                 const int64_t *d_step, int kstep, int rows)
+                 int64_t ny, float ce, float cpe, float ch, float cph, Cpml<float> cin, Source src, int rows)
 {
     PsiOut po{};
     for (int q = 0; q < 12; ++q) po.psi[q] = psi_out[q];
@@ -1052,17 +1024,16 @@ void launch_eh2d(cudaStream_t st, float *const fin[6], float *const fout[6], flo
         const int ktop = cin.L > 0 ? (int)std::min<int64_t>(nseg, cdiv(cin.L, rows) + 1) : 0;
         dim3 g(cdiv(nx, 128 * kEh2W), nseg);
         launch_pdl(k_eh2d_v4, g, dim3(32 * kEh2W), 0, st, fin[FDTD_EZ], fin[FDTD_HX], fin[FDTD_HY], fout[FDTD_EZ],
-                   fout[FDTD_HX], fout[FDTD_HY], nx, ny, rows, ktop, ce, cpe, ch, cph, cin, po, src, d_step, kstep);
+                   fout[FDTD_HX], fout[FDTD_HY], nx, ny, rows, ktop, ce, cpe, ch, cph, cin, po, src);
         return;
     }
     dim3 g(cdiv(nx, kF2X), cdiv(ny, kF2Y));
     launch_pdl(k_eh2d, dim3(g), dim3(kF2T), 0, st, fin[FDTD_EZ], fin[FDTD_HX], fin[FDTD_HY], fout[FDTD_EZ], fout[FDTD_HX], fout[FDTD_HY],
-                               nx, ny, ce, cpe, ch, cph, cin, po, src, d_step, kstep);
+                               nx, ny, ce, cpe, ch, cph, cin, po, src);
 }
 
 void launch_eh3d(cudaStream_t st, float *const fin[6], float *const fout[6], float *const psi_out[12], int64_t nx,
-                 int64_t ny, int64_t nz, float ce, float cpe, float ch, float cph, Cpml<float> cin, Source src,
-                 const int64_t *d_step, int kstep)
+                 int64_t ny, int64_t nz, float ce, float cpe, float ch, float cph, Cpml<float> cin, Source src)
 {
     const int tz = 32;
     dim3 g(cdiv(nx, kEhX), cdiv(ny, kEhY), cdiv(nz, tz));
@@ -1070,7 +1041,7 @@ void launch_eh3d(cudaStream_t st, float *const fin[6], float *const fout[6], flo
     FieldOut o{fout[0], fout[1], fout[2], fout[3], fout[4], fout[5]};
     PsiOut po{};
     for (int q = 0; q < 12; ++q) po.psi[q] = psi_out[q];
-    launch_pdl(k_eh3d, dim3(g), dim3(dim3(kEhX, kEhY)), 0, st, a, o, nx, ny, nz, tz, ce, cpe, ch, cph, cin, po, src, d_step, kstep);
+    launch_pdl(k_eh3d, dim3(g), dim3(dim3(kEhX, kEhY)), 0, st, a, o, nx, ny, nz, tz, ce, cpe, ch, cph, cin, po, src);
 }
 
 

@@ -84,8 +84,9 @@ struct Source {
     int kind, loc;
     double amp, fc, tau, t0, dt;
     int64_t i, j, k, i0, i1, j0, j1;
-    double *val;   // device scalar: g(t^{n+1}) of the current step, written by the H kernel
+    double *val;   // device: g(t^{n+1}) of the step; an H update at step offset 0 writes kSourceSteps of them
 };
+constexpr int kSourceSteps = 32;   // no sequence of steps is longer
 
 // g(t) of the soft source, FP64 on the device
 __device__ __forceinline__ double source_value(const Source &s, double t)
@@ -240,11 +241,9 @@ void launch_e3d(cudaStream_t st, T *const f[6], int64_t nx, int64_t ny, int64_t 
 // 2-D / 3-D FP32 fused E^{n+1} + H^{n+3/2}: read fields fin and psi cin.psi, write fout and psi_out
 // (2-D: rows > 0 with nx a multiple of 4 selects the column march, rows per block segment)
 void launch_eh2d(cudaStream_t st, float *const fin[6], float *const fout[6], float *const psi_out[12], int64_t nx,
-                 int64_t ny, float ce, float cpe, float ch, float cph, Cpml<float> cin, Source src,
-                 const int64_t *d_step, int kstep, int rows);
+                 int64_t ny, float ce, float cpe, float ch, float cph, Cpml<float> cin, Source src, int rows);
 void launch_eh3d(cudaStream_t st, float *const fin[6], float *const fout[6], float *const psi_out[12], int64_t nx,
-                 int64_t ny, int64_t nz, float ce, float cpe, float ch, float cph, Cpml<float> cin, Source src,
-                 const int64_t *d_step, int kstep);
+                 int64_t ny, int64_t nz, float ce, float cpe, float ch, float cph, Cpml<float> cin, Source src);
 void launch_advance(cudaStream_t st, int64_t *d_step, int64_t by);
 // FP32 curl stencils fed by TMA (3-D: 32 x 8 columns walking tz planes along z; 2-D: 32-cell strips
 // walking rows in 16-row chunks); the tensor maps describe one field set (nx a multiple of 4; maps made
@@ -269,7 +268,7 @@ bool tma_fused_prepare(TmaMaps *t, float *const f0[6], float *const f1[6]);
 void tma_fused_forget(TmaMaps *t);
 bool launch_eh3d_tma(cudaStream_t st, const TmaMaps *t, float *const fin[6], float *const fout[6],
                      float *const psi_out[12], float ce, float cpe, float ch, float cph, Cpml<float> cin, Source src,
-                     const int64_t *d_step, int kstep, int tz, int *err);
+                     int tz, int *err);
 
 // GPU compaction of a density array into plasma slots (compact.cu): chunks of kCompactChunk nodes; per
 // chunk the number of plasma nodes and the largest density (bad |= 1 on a non-finite or negative value),
@@ -430,7 +429,7 @@ struct fdtd_plasma {
     int64_t prof_len;
     void *mur_state;
     int64_t *d_step;
-    double *d_src;            // g(t^{n+1}) of the step in flight
+    double *d_src;            // g(t^{n+1}) of the steps of the sequence in flight
     int *d_err;               // device error word (bounded waits that gave up)
     int64_t steps_done;
     // domain decomposition along the slowest axis (fdtd_plasma_create_subdomain; sd_on = 0: a whole grid):

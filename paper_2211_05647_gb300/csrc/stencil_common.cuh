@@ -20,12 +20,40 @@ __device__ __forceinline__ bool in_slab(int64_t i, int64_t n, int L)
     return i < L || i >= n - L;
 }
 
-// g(t^{n+1}) is evaluated once per step, by the first thread of the H kernel,
-// into a device scalar that the E kernel of the same step reads at the source
-// node(s) -- no FP64 transcendental in the E stencil.
-__device__ __forceinline__ void write_source(const Source &src, const int64_t *d_step, int kstep)
+// The source values g(t^{n+1}) of a sequence's steps are evaluated once, by the
+// first warp of its first H launch (kstep 0), a lane a step, into the table the
+// E updates of the sequence read at the source node(s).  The FP64 sin and exp
+// hold the warp for two microseconds whatever the lanes that need them: in every
+// H launch that latency was longer than the rest of a short step's H update
+// (64 x 64 grid with 64-node rows 5.6 -> 4.2 us a step, 512^2 14.4 -> 13.4; where
+// the row kernel's early loads already hid it, as on 192 x 160 with 1024-node
+// rows, nothing changes).
+// Called by the whole first block (t: the thread's index in it, of nt).  Out of
+// line: inlined, its FP64 code raised the H kernels' registers (32 to 40, 40 to
+// 48) and cost them CTAs (3-D cell kernels of odd nx: 4 % of a step).
+static __device__ __noinline__ void eval_sources(double *val, int kind, double amp, double fc, double tau, double t0,
+                                                 double dt, int64_t step, int t, int nt)
 {
-    if (src.kind) *src.val = source_value(src, (double)(*d_step + kstep + 1) * src.dt);
+    Source s{};
+    s.kind = kind;
+    s.amp = amp;
+    s.fc = fc;
+    s.tau = tau;
+    s.t0 = t0;
+    for (; t < kSourceSteps; t += nt) val[t] = source_value(s, (double)(step + t + 1) * dt);
+}
+__device__ __forceinline__ void write_source(const Source &s, const int64_t *d_step, int kstep, int t, int nt)
+{
+    if (s.kind && kstep == 0 && t < kSourceSteps)
+        eval_sources(s.val, s.kind, s.amp, s.fc, s.tau, s.t0, s.dt, *d_step, t, nt);
+}
+
+// the same for the kernels whose blocks are one cell (or four) a thread
+__device__ __forceinline__ void write_source_block0(const Source &src, const int64_t *d_step, int kstep)
+{
+    if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0)
+        write_source(src, d_step, kstep, (threadIdx.z * blockDim.y + threadIdx.y) * blockDim.x + threadIdx.x,
+                     blockDim.x * blockDim.y * blockDim.z);
 }
 
 // Fixed-rounding arithmetic of the 2-D TMz updates.  Every 2-D kernel (one

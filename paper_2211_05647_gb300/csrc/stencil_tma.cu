@@ -120,7 +120,7 @@ __global__ void __launch_bounds__(kTT, kMinBlocks) k_h3d_tma(const __grid_consta
     const int64_t i = x0 + tx, j = y0 + ty;
     const bool own = i < nx && j < ny;
     if (quit_early(err, &s.quit)) return;   // an earlier block's wait gave up: the step is void
-    if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && tid == 0) write_source(src, d_step, kstep);
+    write_source_block0(src, d_step, kstep);
     if (tid == 0) {
         for (int q = 0; q < kStages; ++q) mbar_init(&s.full[q], 1);
         fence_proxy_async_smem();
@@ -302,7 +302,7 @@ __device__ __forceinline__ bool source_column(const Source &src, int64_t i, int6
 __global__ void __launch_bounds__(kTT, kFMinBlocks) k_eh3d_tma(const __grid_constant__ FusedBoxes bx, FusedOut out,
                                                               int nx, int ny, int nz, int tz, float ce, float cpe,
                                                               float ch, float cph, Cpml<float> cin, Source src,
-                                                              const int64_t *__restrict__ d_step, int kstep, int *err)
+                                                              int *err)
 {
     extern __shared__ __align__(128) float ring[];
     float *ebuf = ring + kFStages * kFStage;   // [2][3][kFBuf]: E^{n+1} of planes of even / odd z
@@ -314,10 +314,7 @@ __global__ void __launch_bounds__(kTT, kFMinBlocks) k_eh3d_tma(const __grid_cons
     const int zs = z0 > 0 ? z0 - 1 : 0, ze = z1 < nz ? z1 : z1 - 1, np = ze - zs + 1;
     if (quit_early(err, &s.quit)) return;
     if (tid == 0) {
-        const int64_t n1 = *d_step + kstep + 1;   // E^{n+1} is at t^{n+1}
-        s_g = src.kind && src.k >= zs && src.k <= ze ? (float)source_value(src, (double)n1 * src.dt) : 0.f;
-        if (src.kind && blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0)
-            *src.val = source_value(src, (double)(n1 + 1) * src.dt);   // for an unfused E update that follows
+        s_g = src.kind ? (float)*src.val : 0.f;
         for (int q = 0; q < kFStages; ++q) mbar_init(&s.full[q], 1);
         fence_proxy_async_smem();
         for (int p = 0; p < min(kFStages, np); ++p) issue_fused_plane(bx, ring, s.full, p, x0, y0, zs + p);
@@ -459,7 +456,7 @@ __global__ void __launch_bounds__(kTT, kMinBlocks) k_h2d_tma(const __grid_consta
     const int np = (min(rows, ny - y0) + kC2 - 1) / kC2;   // chunks
     const int64_t i = x0 + tx;
     if (quit_early(err, &s.quit)) return;
-    if (blockIdx.x == 0 && blockIdx.y == 0 && tid == 0) write_source(src, d_step, kstep);
+    write_source_block0(src, d_step, kstep);
     auto issue = [&](int p) {
         float *st = ring + (p % kS2Stages) * kS2H;
         uint64_t *m = &s.full[p % kS2Stages];
@@ -732,7 +729,7 @@ void launch_h3d_tma(cudaStream_t st, const TmaMaps *t, float *const f[6], int64_
 
 bool launch_eh3d_tma(cudaStream_t st, const TmaMaps *t, float *const fin[6], float *const fout[6],
                      float *const psi_out[12], float ce, float cpe, float ch, float cph, Cpml<float> cin, Source src,
-                     const int64_t *d_step, int kstep, int tz, int *err)
+                     int tz, int *err)
 {
     if (!t || !t->fused_ready) return false;
     int b = -1;
@@ -747,7 +744,7 @@ bool launch_eh3d_tma(cudaStream_t st, const TmaMaps *t, float *const fin[6], flo
     if (!attr) return false;
     const dim3 g(cdivu(t->nx, kTX), cdivu(t->ny, kTY), cdivu(t->nz, tz));
     launch_plain(k_eh3d_tma, dim3(g), dim3(kTT), kFSmemBytes, st, t->fused[b], o, (int)t->nx, (int)t->ny, (int)t->nz, tz, ce, cpe, ch, cph,
-                                            cin, src, d_step, kstep, err);
+                                            cin, src, err);
     return true;
 }
 
