@@ -40,7 +40,7 @@ __global__ void __launch_bounds__(256) k_kinetic(KinArgs<TA> a)
     if (kEarly && row < a.nslots) {
         const V *rp = reinterpret_cast<const V *>(a.df) + row * (a.pitch / VEC);
 #pragma unroll
-        for (int q = 0; q < VPL; ++q) v[q] = __ldcs(rp + q * L + l);
+        for (int q = 0; q < VPL; ++q) v[q] = __ldcg(rp + q * L + l);   // (from L2, where the writes are)
     }
     __syncthreads();
     pdl_enter();
