@@ -36,6 +36,12 @@ __global__ void __launch_bounds__(256) k_kinetic(KinArgs<TA> a)
     int32_t cell_next = row < a.nslots ? __ldg(a.slot_cell + row) : 0;
     // (not the shortest BF16 rows: one more condition in their loop costs them a CTA a SM and 10 %)
     constexpr bool kEarly = !(std::is_same<TS, __nv_bfloat16>::value && VPL * L <= 8);
+    // Rows a lane each: consecutive vectors share a 32-byte sector, so the lines stay in L1 by the plain policy until
+    // the row is loaded (streaming loads give them up early: 32-node BF16 rows, 2 GB of them 755 -> 721 us, 16-node
+    // FP32 rows 841 -> 793, 16-node BF16 rows 808 -> 792).  Two-vector FP32 rows and longer rows are no faster with it
+    // (8-node FP32 789 -> 821, 64-node BF16 709 -> 710) and keep the streaming hint.
+    constexpr bool kShared = L == 1 && !std::is_same<TS, double>::value &&
+                             (VPL == 4 || (VPL == 2 && std::is_same<TS, __nv_bfloat16>::value));
     V v[VPL];
     if (kEarly && row < a.nslots) {
         const V *rp = reinterpret_cast<const V *>(a.df) + row * (a.pitch / VEC);
@@ -55,7 +61,7 @@ __global__ void __launch_bounds__(256) k_kinetic(KinArgs<TA> a)
         if (valid) {
             if (!kEarly || !loaded) {
 #pragma unroll
-                for (int q = 0; q < VPL; ++q) v[q] = __ldcs(rp + q * L + l);
+                for (int q = 0; q < VPL; ++q) v[q] = kShared ? rp[q * L + l] : __ldcs(rp + q * L + l);
             }
             E = a.E[cell];
             nE = __ldg(a.dens + row) * E;
