@@ -1863,9 +1863,11 @@ int autotune_t(fdtd_plasma *h, fdtd_tune_result *out)
         int cand[8][2];
         const int nc = kinetic_candidates(h->pitch, h->pl.f_dtype, cand);
         // (ring stages, CTAs per SM cap): the register kernel, then the bulk-copy ring (FP32 / BF16 rows).
-        // Each candidate is timed where it runs, between the H and E stencils of whole steps (events around
-        // the middle part, as fdtd_plasma_time_kernels does): timed back to back on their own, some ring
-        // shapes that lose inside the step looked fastest.
+        // Each candidate is timed where it runs: a sequence of whole steps, with the stencil passes chosen above
+        // and no events inside.  Timed back to back on their own, some ring shapes that lose inside the step
+        // looked fastest; timed by events around the middle part, the register kernel looked within 1 % of the
+        // ring (4096^2, 1024-node rows: 1.011 against 1.001 ms) and was kept half the time, at 1.127 against
+        // 1.074 ms a step.
         static const int variants[][2] = {{0, 0}, {0, 2}, {0, 3}, {2, 0}, {3, 0}, {4, 0}, {6, 0}};
         cudaEvent_t ev[5];
         for (int q = 0; q < 5; ++q) CK(h, cudaEventCreate(&ev[q]));
@@ -1885,6 +1887,19 @@ int autotune_t(fdtd_plasma *h, fdtd_tune_result *out)
             }
             return acc / 5.0;
         };
+        auto time_steps = [&](bool &bad) -> double {
+            constexpr int n = 7;   // six transitions, all fused where the steps fuse
+            for (int r = 0; r < 2 && !bad; ++r) {
+                if (r) cudaEventRecord(ev[0], st);
+                bad = enqueue_seq<T>(h, st, r ? n : 1) != cudaSuccess;
+            }
+            cudaEventRecord(ev[1], st);
+            float ms = 0;
+            if (cudaEventSynchronize(ev[1]) != cudaSuccess || cudaEventElapsedTime(&ms, ev[0], ev[1]) != cudaSuccess)
+                bad = true;
+            if (bad) cudaGetLastError();
+            return ms / n;
+        };
         const int keep[3] = {h->kin_vpl, h->kin_l, h->kin_bps}, keep_stages = h->kin_stages;
         // the timing steps leave no trace outside the saved state: no port spectra, no recorded samples
         const int keep_ports = h->nports, keep_rec = h->has_recording;
@@ -1898,23 +1913,24 @@ int autotune_t(fdtd_plasma *h, fdtd_tune_result *out)
                     continue;
                 bool bad = false;
                 h->kin_vpl = cand[c][0]; h->kin_l = cand[c][1]; h->kin_bps = vr[1]; h->kin_stages = vr[0];
-                const double ms = time_in_step(bad);
+                const double ms = time_steps(bad);
                 if (!bad && ms < best * kTuneMargin) {
                     best = ms;
                     out->kin_vpl = cand[c][0]; out->kin_l = cand[c][1]; out->kin_blocks_per_sm = vr[1];
                     out->kin_stages = vr[0];
                 }
             }
-        for (int q = 0; q < 5; ++q) cudaEventDestroy(ev[q]);
-        h->nports = keep_ports;
-        h->has_recording = keep_rec;
         if (best >= 1e30) {   // nothing ran: keep the shape in use
             out->kin_vpl = keep[0]; out->kin_l = keep[1]; out->kin_blocks_per_sm = keep[2];
             out->kin_stages = keep_stages;
         }
         h->kin_vpl = out->kin_vpl; h->kin_l = out->kin_l; h->kin_bps = out->kin_blocks_per_sm;
         h->kin_stages = out->kin_stages;
-        out->kin_ms = best;
+        bool bad = best >= 1e30;
+        out->kin_ms = bad ? best : time_in_step(bad);   // per launch
+        for (int q = 0; q < 5; ++q) cudaEventDestroy(ev[q]);
+        h->nports = keep_ports;
+        h->has_recording = keep_rec;
         m[kin_key(h)] = {out->kin_vpl, out->kin_l, out->kin_blocks_per_sm, out->kin_stages};
     }
     cudaEventDestroy(e0);
