@@ -15,7 +15,7 @@
 // sixteen: kinetic_default_shape); a warp covers 32/L rows.  The whole row is loaded
 // before any arithmetic so each lane has VPL 16-byte loads in flight, the
 // loads/stores use the streaming (evict-first) cache hint because delta f is
-// far larger than L2, and the per-node tables sit in shared memory.
+// far larger than L2 (rows of one lane each load without it: k_kinetic), and the per-node tables sit in shared memory.
 // BF16 storage: FP32 arithmetic, stochastic rounding on store with 16 random
 // bits per node from Philox4x32-7 keyed by the seed and counted by
 // (slot, vector, step).
