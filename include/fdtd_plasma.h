@@ -296,8 +296,8 @@ int fdtd_selftest_timed_wait(uint32_t limit_us, int32_t *gave_up);
  * delta f.  The order J is summed in follows (vpl, l).
  * Needs a plasma (after set_plasma).  The autotuner overwrites it.
  * FDTD_OPT_FUSED_ROWS (2-D fused pass, nx a multiple of 4): rows per block
- * segment of the column-march kernel (1..4096, default 8; each warp owns a
- * 128-column strip and marches up the segment with no shared memory); 0
+ * segment of the column-march kernel (1..4096, default 8, at least ny / 65535;
+ * each warp owns a 128-column strip and marches up the segment with no shared memory); 0
  * selects the 64 x 16 shared-memory tiles instead.  Both equal the unfused
  * sequence up to FP32 rounding order.
  * FDTD_ERR_INVAL for an unknown option or value. */

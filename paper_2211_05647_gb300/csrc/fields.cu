@@ -1020,6 +1020,7 @@ void launch_eh2d(cudaStream_t st, float *const fin[6], float *const fout[6], flo
     PsiOut po{};
     for (int q = 0; q < 12; ++q) po.psi[q] = psi_out[q];
     if (rows > 0 && nx % 4 == 0 && ny < (int64_t(1) << 31)) {   // the column march (16-byte rows, 32-bit row index)
+        rows = std::max<int>(rows, (int)cdiv(ny, 65535));        // segments lie in the grid's y dimension
         const unsigned nseg = cdiv(ny, rows);
         const int ktop = cin.L > 0 ? (int)std::min<int64_t>(nseg, cdiv(cin.L, rows) + 1) : 0;
         dim3 g(cdiv(nx, 128 * kEh2W), nseg);

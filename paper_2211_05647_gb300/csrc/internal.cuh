@@ -239,7 +239,8 @@ template <typename T>
 void launch_e3d(cudaStream_t st, T *const f[6], int64_t nx, int64_t ny, int64_t nz, T ce, T cpe, Cpml<T> cp,
                 Source src, const int64_t *d_step, int kstep, dim3 block, int cpt);
 // 2-D / 3-D FP32 fused E^{n+1} + H^{n+3/2}: read fields fin and psi cin.psi, write fout and psi_out
-// (2-D: rows > 0 with nx a multiple of 4 selects the column march, rows per block segment)
+// (2-D: rows > 0 with nx a multiple of 4 selects the column march, rows per block segment, more where ny has more
+// than 65535 segments)
 void launch_eh2d(cudaStream_t st, float *const fin[6], float *const fout[6], float *const psi_out[12], int64_t nx,
                  int64_t ny, float ce, float cpe, float ch, float cph, Cpml<float> cin, Source src, int rows);
 void launch_eh3d(cudaStream_t st, float *const fin[6], float *const fout[6], float *const psi_out[12], int64_t nx,

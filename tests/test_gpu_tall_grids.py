@@ -1,0 +1,40 @@
+"""Long, narrow FP32 grids, whose block counts along y or z come near the 65535 of a launch: every stencil path the
+size rules or an option can choose gives the grid-of-cells kernels' fields bit for bit."""
+import numpy as np
+import pytest
+
+from tests.adapters import FIELDS
+
+pytestmark = pytest.mark.gpu
+
+
+def _start(dims, cpml):
+    from paper_2211_05647_gb300 import Solver
+    nx, ny, nz = (*dims, 1)[:3]
+    nd = len(dims)
+    s = Solver(dict(ndim=nd, nx=nx, ny=ny, nz=nz, dx=1e-3, courant=0.5, cpml_cells=cpml, mur=0, precision="f32"))
+    s.set_source(kind="gauss", amp=1.0, tau=1e-11, t0=0.0, i=nx // 2, j=ny // 2, k=nz // 2)
+    rng = np.random.default_rng(3)
+    for q in FIELDS[nd]:
+        s.write(q, rng.standard_normal(nx * ny * nz, dtype=np.float32) / (1.0 if q[0] == "e" else 377.0))
+    return s
+
+
+def _equal(a, b, nd):
+    for k in (1, 4, 7):
+        a.step(k)
+        b.step(k)
+    assert all(np.array_equal(a.read(q, device=False), b.read(q, device=False)) for q in FIELDS[nd])
+
+
+@pytest.mark.parametrize("dims,cpml,rows", [((24, 262144), 4, None), ((24, 262140), 4, None), ((8, 262141), 2, 4),
+                                            ((8, 65537), 2, 1)])
+def test_march_on_tall_grids(dims, cpml, rows):
+    """6.3 M cells take the fused march by the size rule; shorter ones by option with the given rows a segment."""
+    a, b = _start(dims, cpml), _start(dims, cpml)
+    b.set_option("stencil_tz", 0)
+    if rows:
+        a.set_option("fused_stencils", 1)
+        a.set_option("fused_rows", rows)
+    assert a.launch_shapes()["fused_rows"] > 0 and b.launch_shapes()["fused_rows"] == 0
+    _equal(a, b, 2)
