@@ -363,8 +363,7 @@ void default_stencils(fdtd_plasma *h)
         h->auto_fuse_rows = cells >= 32000000 ? 8 : 4;
         h->fuse_by_rule = 1;
     } else if (h->g.ndim == 3 && cells >= 12000000) {
-        h->st_tz = 12;
-        h->st_bx = 32; h->st_by = 8; h->st_bz = 1; h->st_cpt = 1;
+        h->st_tz = 12;   // (the grid-of-cells block keeps its default, for when the option turns the columns off)
     }
 }
 

@@ -38,3 +38,14 @@ def test_march_on_tall_grids(dims, cpml, rows):
         a.set_option("fused_rows", rows)
     assert a.launch_shapes()["fused_rows"] > 0 and b.launch_shapes()["fused_rows"] == 0
     _equal(a, b, 2)
+
+
+@pytest.mark.parametrize("dims", [(16, 12, 65537), (16, 12, 66000)])
+def test_cell_kernels_on_deep_grids(dims):
+    """12.6 M cells take the TMA columns by the size rule; turned off, the grid-of-cells kernels cover two planes a
+    block, as they do on grids the rule leaves alone (one plane a block would need more than 65535 along z)."""
+    a, b = _start(dims, 2), _start(dims, 2)
+    b.set_option("stencil_tz", 0)
+    assert a.launch_shapes()["stencil_tz"] > 0 and b.launch_shapes()["stencil_tz"] == 0
+    assert b.launch_shapes()["block_z"] == 2
+    _equal(a, b, 3)
