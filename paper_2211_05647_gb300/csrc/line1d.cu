@@ -335,39 +335,4 @@ size_t line1d_smem_bytes(int f_dtype, int pitch, int rows, int nodes)
     return LineSmem<float, float>(pitch, rows, nodes).total;
 }
 
-// Equal-cost contiguous ranges of the nodes 0 .. nz for `ctas` CTAs (fewer when the line is short: four nodes
-// or more each): cut[c] the first node of range c, slot_cut[c] its first plasma slot.  Node 0 shares a range
-// with node 1 and node nz with node nz - 1 (the Mur ends).  A row costs row_cost nodes.
-LinePlan line1d_plan(int64_t nz, const std::vector<int32_t> &cells, int ctas, double row_cost)
-{
-    LinePlan p;
-    const int64_t n = nz + 1, ns = (int64_t)cells.size();
-    const int64_t want = std::max<int64_t>(1, std::min<int64_t>(ctas, n / 4));
-    const double total = (double)n + row_cost * (double)ns;
-    p.cut.push_back(0);
-    p.slot_cut.push_back(0);
-    double acc = 0.0;
-    int64_t s = 0;
-    for (int64_t k = 0; k < n; ++k) {
-        acc += 1.0;
-        if (s < ns && cells[(size_t)s] == k) {
-            acc += row_cost;
-            ++s;
-        }
-        const int64_t c = k + 1;   // a cut after node k
-        const double target = total * (double)p.cut.size() / (double)want;
-        if ((int64_t)p.cut.size() < want && acc >= target && c >= 2 && c <= nz - 1) {
-            p.cut.push_back((int32_t)c);
-            p.slot_cut.push_back((int32_t)s);
-        }
-    }
-    p.cut.push_back((int32_t)n);
-    p.slot_cut.push_back((int32_t)ns);
-    for (size_t c = 0; c + 1 < p.cut.size(); ++c) {
-        p.nodes_max = std::max(p.nodes_max, p.cut[c + 1] - p.cut[c]);
-        p.rows_max = std::max(p.rows_max, p.slot_cut[c + 1] - p.slot_cut[c]);
-    }
-    return p;
-}
-
 }  // namespace fp

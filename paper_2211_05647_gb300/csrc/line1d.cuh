@@ -1,10 +1,8 @@
 // line1d.cuh -- interface of the 1-D cooperative stepping kernel (line1d.cu).
 #pragma once
 
-#include <algorithm>
-#include <vector>
-
 #include "internal.cuh"
+#include "line_plan.cuh"
 
 namespace fp {
 
@@ -25,11 +23,6 @@ struct LineArgs {
     TA ch, ce, cj, m;
 };
 
-struct LinePlan {
-    std::vector<int32_t> cut, slot_cut;   // range starts, one more than there are CTAs
-    int nodes_max = 0, rows_max = 0;
-};
-LinePlan line1d_plan(int64_t nz, const std::vector<int32_t> &cells, int ctas, double row_cost);
 size_t line1d_smem_bytes(int f_dtype, int pitch, int rows, int nodes);
 template <typename TA>
 cudaError_t launch_line1d(cudaStream_t st, const LineArgs<TA> &a, int f_dtype, int ctas);
