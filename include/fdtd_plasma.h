@@ -210,10 +210,13 @@ int fdtd_plasma_time_kernels(fdtd_plasma_t h, int64_t nsteps, double *ms_out);
  * keyed by GPU name, kernel, precision and size class; later handles of the
  * same class start from the cached shapes.  The state is saved before and
  * restored bit for bit after (needs one temporary copy of it on the device).
- * Synchronous. */
+ * A 1-D grid that fdtd_plasma_step takes in one cooperative launch runs
+ * neither kernel: nothing is timed there, no cached shape applies, and a shape
+ * set by FDTD_OPT_KINETIC_SHAPE goes back to the default.  Synchronous. */
 typedef struct {
     int32_t kin_vpl, kin_l, kin_blocks_per_sm;   /* 0 = no kinetic kernel tuned */
-    int32_t block_x, block_y, block_z;           /* 0 = no stencil tuned (1-D) */
+    int32_t block_x, block_y, block_z;           /* 0 = no stencil tuned (1-D; of launch_shapes: the threads of the
+                                                    1-D cooperative kernel when it steps the grid, else 0) */
     double kin_ms, stencil_ms;                   /* best per-launch times */
     int32_t cells_per_thread;                    /* stencils: 1, or 4 (FP32 rows of a multiple of 4 cells;
                                                     block_x then counts groups of 4 cells) */
@@ -293,7 +296,10 @@ int fdtd_selftest_timed_wait(uint32_t limit_us, int32_t *gave_up);
  * register kernel) or 2..64 (the bulk-copy ring kernel: FP32 / BF16 rows of
  * the linear update, stages that fit in one CTA's shared memory); 0 returns
  * to the built-in default, which follows the row's length and the bytes of
- * delta f.  The order J is summed in follows (vpl, l).
+ * delta f.  The order J is summed in follows (vpl, l): a 1-D grid is then
+ * stepped by graphs of that kernel unless the cooperative one sums FP32 or BF16
+ * rows in this order (the default's; its FP64 rows differ from those of
+ * time_kernels by roundings of J).
  * Needs a plasma (after set_plasma).  The autotuner overwrites it.
  * FDTD_OPT_FUSED_ROWS (2-D fused pass, nx a multiple of 4): rows per block
  * segment of the column-march kernel (1..4096, default 8, at least ny / 65535;

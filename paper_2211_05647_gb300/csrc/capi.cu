@@ -554,6 +554,20 @@ cudaError_t part_h(fdtd_plasma *h, cudaStream_t st, int kstep, const FieldSet<T>
     return cudaGetLastError();
 }
 
+bool line_steps(fdtd_plasma *h);
+
+// the kinetic row shape in use (0: the built-in default).  A grid that the 1-D stepping kernel steps has the default
+// unless the option asked for another: a tuned shape is the row kernel's, and J must not be summed in one order by
+// step and in another by time_kernels
+struct KinShape {
+    int vpl, l, bps, stages;
+};
+KinShape kin_shape(fdtd_plasma *h)
+{
+    if (!h->kin_forced && line_steps(h)) return {0, 0, 0, 0};
+    return {h->kin_vpl, h->kin_l, h->kin_bps, h->kin_stages};
+}
+
 // the work between the H and E updates: E-history push, kinetic update (E -= dt/eps0 J), closure, recorder.
 // J^{n+1/2} per slot is stored on the last step of a sequence (what read_fields and checkpoints see between
 // step calls) and on every step while the recorder, which reads it, is on.  after_stencil: no call can come
@@ -592,7 +606,8 @@ cudaError_t part_mid(fdtd_plasma *h, cudaStream_t st, int kstep, const FieldSet<
             const int nperp = h->pl.vgrid == FDTD_VGRID_CART2D ? h->pl.nv_perp : 1;
             e = launch_kinetic_nl<T>(st, a, h->pl.nv, nperp, dvpar, kQe / kMe, h->dt, h->num_sms);
         } else {
-            e = launch_kinetic<T>(st, a, h->pl.f_dtype, h->num_sms, h->kin_vpl, h->kin_l, h->kin_bps, h->kin_stages);
+            const KinShape k = kin_shape(h);
+            e = launch_kinetic<T>(st, a, h->pl.f_dtype, h->num_sms, k.vpl, k.l, k.bps, k.stages);
         }
         if (e != cudaSuccess) return e;
     }
@@ -799,24 +814,55 @@ cudaError_t enqueue(fdtd_plasma *h, cudaStream_t st, int nsteps)
 // the step graphs.  Measured against the graphs over the sizes that fit: 500 rows of 64 nodes on 2000 cells, FP32
 // 0.97 against 6.0 us a step, FP64 2.3 against 13.1; 30 k rows, FP32 4.9 against 8.0; 100 k BF16 rows 11.6 both
 // (FP32: no longer fits); a million cells without plasma 2.6 against 8.7.  So what fits takes the kernel.
+// A row shape asked for by option sums J in its own order: only where that is the order of the kernel's rows (the
+// default shape's; in FP64 rows they have a shape of their own) does the kernel take the grid.
 bool line_applies(const fdtd_plasma *h)
 {
     if (h->g.ndim != 1 || h->nports > 0 || h->has_recording || h->has_closure) return false;
-    return !(h->has_plasma && (h->pl.nonlinear || h->pl.evolve_f0));
+    if (!h->has_plasma) return true;
+    if (h->pl.nonlinear || h->pl.evolve_f0) return false;
+    if (!h->kin_forced) return true;
+    int vpl = 0, l = 0;
+    kinetic_default_shape(h->pitch, h->pl.f_dtype, &vpl, &l);
+    return h->pl.f_dtype != FDTD_DF_F64 && h->kin_vpl == vpl && h->kin_l == l;
 }
 
-int line_plan(fdtd_plasma *h)
+// the storage type and row length the kernel is instantiated for (a grid without plasma: no rows)
+int line_dtype(const fdtd_plasma *h)
 {
-    h->line_state = -1;
-    const int f_dtype = h->g.precision == FDTD_F64 ? FDTD_DF_F64 : (h->has_plasma ? h->pl.f_dtype : FDTD_DF_F32);
-    const int pitch = h->has_plasma ? h->pitch : 0, vec = f_dtype == FDTD_DF_BF16 ? 8 : (f_dtype == FDTD_DF_F64 ? 2 : 4);
-    if (pitch / vec > 128) return FDTD_OK;
+    return h->g.precision == FDTD_F64 ? FDTD_DF_F64 : (h->has_plasma ? h->pl.f_dtype : FDTD_DF_F32);
+}
+
+LinePlan line_plan(const fdtd_plasma *h)
+{
     // a row weighs its nodes: an FP64 row is bound by the FP64 pipe, and the cells of a range cost next to nothing
-    const LinePlan p = line1d_plan(h->nz, h->h_cells, h->num_sms, (double)pitch);
-    int dev = 0, most = 0;
-    CK(h, cudaGetDevice(&dev));
-    CK(h, cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev));
-    if (line1d_smem_bytes(f_dtype, pitch, p.rows_max, p.nodes_max) + 1024 > (size_t)most) return FDTD_OK;
+    return line1d_plan(h->nz, h->h_cells, h->num_sms, h->has_plasma ? (double)h->pitch : 0.0);
+}
+
+// whether the 1-D stepping kernel steps the grid, decided from sizes alone on first use
+bool line_steps(fdtd_plasma *h)
+{
+    if (!line_applies(h)) return false;
+    if (h->line_state == 0) {
+        h->line_state = -1;
+        const int f_dtype = line_dtype(h), pitch = h->has_plasma ? h->pitch : 0;
+        if (pitch / (f_dtype == FDTD_DF_BF16 ? 8 : (f_dtype == FDTD_DF_F64 ? 2 : 4)) > 128) return false;
+        const LinePlan p = line_plan(h);
+        int dev = 0, most = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        if (line1d_smem_bytes(f_dtype, pitch, p.rows_max, p.nodes_max) + 1024 <= (size_t)most) h->line_state = 1;
+    }
+    return h->line_state > 0;
+}
+
+// the plan and the mailboxes on the device, before the first launch
+int line_prepare(fdtd_plasma *h)
+{
+    const LinePlan p = line_plan(h);
     const size_t n = p.cut.size();
     h->line_cut = (int32_t *)dalloc(h, 2 * n * sizeof(int32_t));
     h->line_mail = (uint64_t *)dalloc(h, (n - 1) * 8 * sizeof(uint64_t));
@@ -835,7 +881,6 @@ int line_plan(fdtd_plasma *h)
     h->line_rows = p.rows_max;
     h->line_nodes = p.nodes_max;
     h->line_seq = 1;
-    h->line_state = 1;
     return FDTD_OK;
 }
 
@@ -872,8 +917,7 @@ cudaError_t line_launch(fdtd_plasma *h, int nsteps)
     a.ce = (T)(h->dt / (kEps0 * h->g.dx));
     a.cj = (T)(h->dt / kEps0);
     a.m = (T)((kC0 * h->dt - h->g.dx) / (kC0 * h->dt + h->g.dx));
-    return launch_line1d<T>(h->stream, a, h->has_plasma ? h->pl.f_dtype : (sizeof(T) == 8 ? FDTD_DF_F64 : FDTD_DF_F32),
-                            h->line_ctas);
+    return launch_line1d<T>(h->stream, a, line_dtype(h), h->line_ctas);
 }
 
 int line_step(fdtd_plasma *h, int64_t nsteps)
@@ -1199,6 +1243,7 @@ int fdtd_plasma_set_option(fdtd_plasma_t h, int option, int64_t value)
         h->kin_l = l;
         h->kin_bps = bps;
         h->kin_stages = stages;
+        h->kin_forced = value != 0;
         return FDTD_OK;
     }
     return fail(h, FDTD_ERR_INVAL, "unknown option %d", option);
@@ -1208,11 +1253,15 @@ int fdtd_plasma_launch_shapes(fdtd_plasma_t h, fdtd_tune_result *out)
 {
     if (!h || !out) return FDTD_ERR_INVAL;
     *out = fdtd_tune_result{};
-    out->kin_vpl = h->kin_vpl;
-    out->kin_l = h->kin_l;
-    out->kin_blocks_per_sm = h->kin_bps;
-    out->kin_stages = h->kin_stages;
-    if (h->g.ndim >= 2) {
+    const KinShape k = kin_shape(h);
+    out->kin_vpl = k.vpl;
+    out->kin_l = k.l;
+    out->kin_blocks_per_sm = k.bps;
+    out->kin_stages = k.stages;
+    if (line_steps(h)) {
+        out->block_x = kLineThreads;
+        out->block_y = out->block_z = 1;
+    } else if (h->g.ndim >= 2) {
         const dim3 b = stencil_block(h);
         out->block_x = (int32_t)b.x; out->block_y = (int32_t)b.y; out->block_z = (int32_t)b.z;
         out->cells_per_thread = stencil_cpt(h);
@@ -1449,7 +1498,7 @@ int fdtd_plasma_set_plasma(fdtd_plasma_t h, const fdtd_plasma_desc *p)
     h->has_plasma = 1;
     h->slot_base = slot_base;
     h->nkin = (int64_t)ns;
-    h->kin_vpl = h->kin_l = h->kin_bps = h->kin_stages = 0;
+    h->kin_vpl = h->kin_l = h->kin_bps = h->kin_stages = h->kin_forced = 0;
     apply_cached_kinetic(h);
     if (ns && dev_slots.p) {   // device to device from the compaction (densities converted to FP32 there)
         const double *d_dens = static_cast<const double *>(dev_slots.p);
@@ -1498,9 +1547,9 @@ int fdtd_plasma_step(fdtd_plasma_t h, int64_t nsteps)
     if (h->sd_on && (h->sd_lo || h->sd_hi || h->sd_half))
         return fail(h, FDTD_ERR_STATE, "a sub-domain with neighbours steps by fdtd_plasma_step_half, exchanging halos");
     if (nsteps == 0) return FDTD_OK;
-    if (line_applies(h)) {
-        if (h->line_state == 0) {
-            const int rc = line_plan(h);
+    if (line_steps(h)) {
+        if (!h->line_cut) {
+            const int rc = line_prepare(h);
             if (rc != FDTD_OK) return rc;
         }
         if (h->line_state > 0) return line_step(h, nsteps);
@@ -1858,7 +1907,10 @@ int autotune_t(fdtd_plasma *h, fdtd_tune_result *out)
     }
     out->kin_vpl = out->kin_l = out->kin_blocks_per_sm = out->kin_stages = 0;
     out->kin_ms = 0;
-    if (h->has_plasma && h->nkin > 0 && !h->pl.nonlinear && !h->pl.evolve_f0) {
+    if (h->has_plasma) h->kin_forced = 0;   // the tuner overwrites the option's shape
+    if (line_steps(h)) {
+        h->kin_vpl = h->kin_l = h->kin_bps = h->kin_stages = 0;   // the row kernel steps nothing here
+    } else if (h->has_plasma && h->nkin > 0 && !h->pl.nonlinear && !h->pl.evolve_f0) {
         int cand[8][2];
         const int nc = kinetic_candidates(h->pitch, h->pl.f_dtype, cand);
         // (ring stages, CTAs per SM cap): the register kernel, then the bulk-copy ring (FP32 / BF16 rows).

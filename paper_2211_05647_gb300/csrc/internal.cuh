@@ -462,6 +462,7 @@ struct fdtd_plasma {
     // launch shapes (autotuner / cache): kinetic (vectors per lane, lanes per row, CTAs per SM; 0 = default),
     // stencil block (0 = default)
     int kin_vpl, kin_l, kin_bps, kin_stages;   // kinetic launch shape; kin_stages > 0: the bulk-copy ring kernel
+    int kin_forced;           // the shape was asked for by FDTD_OPT_KINETIC_SHAPE
     int st_bx, st_by, st_bz, st_cpt;
     int st_tz;                // > 0: 3-D FP32 stencils run the TMA column kernels with tz planes per block
     fp::TmaMaps *tma;         // their tensor maps (field set 0), made on first use
@@ -480,7 +481,7 @@ struct fdtd_plasma {
     int gk_steps;
     int graphs_valid;
     // the 1-D cooperative stepping kernel (line1d.cu): ranges and mailboxes, made on the first step
-    // (line_state 0: not looked at yet, 1: in use, -1: this configuration takes the step graphs)
+    // (line_state 0: not looked at yet, 1: the state fits, -1: this configuration takes the step graphs)
     int line_state, line_ctas, line_rows, line_nodes;
     uint32_t line_seq;         // tag of the next launch's first message
     int32_t *line_cut;         // cut[line_ctas + 1], then slot_cut[line_ctas + 1]

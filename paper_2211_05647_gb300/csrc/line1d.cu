@@ -37,7 +37,6 @@ namespace fp {
 
 namespace {
 
-constexpr int kLineThreads = 512;
 constexpr int kLineWarps = kLineThreads / 32;
 constexpr int kRowWarps = kLineWarps - 2;          // the last two warps take the neighbours' messages
 constexpr int kSrcChunk = 64;                      // source values formed at a time, one a thread

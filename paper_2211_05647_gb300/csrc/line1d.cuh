@@ -6,6 +6,8 @@
 
 namespace fp {
 
+constexpr int kLineThreads = 512;
+
 template <typename TA>
 struct LineArgs {
     TA *E, *H, *mur, *jslot;   // mur == nullptr: PEC ends
