@@ -922,11 +922,6 @@ cudaError_t line_launch(fdtd_plasma *h, int nsteps)
 
 int line_step(fdtd_plasma *h, int64_t nsteps)
 {
-    // the launch carries the step and message counters as arguments: it is not for replay in a caller's graph
-    // (the step graphs cannot be captured either)
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    CK(h, cudaStreamIsCapturing(h->stream, &cs));
-    if (cs != cudaStreamCaptureStatusNone) return cuda_fail(h, cudaErrorStreamCaptureUnsupported, "fdtd_plasma_step");
     for (int64_t left = nsteps; left > 0;) {
         const int n = (int)std::min<int64_t>(left, 65536);
         const cudaError_t e = h->g.precision == FDTD_F64 ? line_launch<double>(h, n) : line_launch<float>(h, n);
@@ -1548,6 +1543,12 @@ int fdtd_plasma_step(fdtd_plasma_t h, int64_t nsteps)
         return fail(h, FDTD_ERR_STATE, "a sub-domain with neighbours steps by fdtd_plasma_step_half, exchanging halos");
     if (nsteps == 0) return FDTD_OK;
     if (line_steps(h)) {
+        // the launch carries the step and message counters as arguments: it is not for replay in a caller's graph
+        // (the step graphs cannot be captured either).  Asked before anything is put on the stream.
+        cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+        CK(h, cudaStreamIsCapturing(h->stream, &cs));
+        if (cs != cudaStreamCaptureStatusNone)
+            return cuda_fail(h, cudaErrorStreamCaptureUnsupported, "fdtd_plasma_step");
         if (!h->line_cut) {
             const int rc = line_prepare(h);
             if (rc != FDTD_OK) return rc;
