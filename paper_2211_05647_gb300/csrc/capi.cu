@@ -19,6 +19,7 @@
 
 #include <sys/stat.h>
 
+#include <cuda.h>
 #include <nvtx3/nvToolsExt.h>
 
 #include "internal.cuh"
@@ -833,10 +834,35 @@ int line_dtype(const fdtd_plasma *h)
     return h->g.precision == FDTD_F64 ? FDTD_DF_F64 : (h->has_plasma ? h->pl.f_dtype : FDTD_DF_F32);
 }
 
+// SMs the handle's stream may use: the device's, or fewer on a stream of a green context
+int stream_sms(const fdtd_plasma *h)
+{
+    using StreamGreen = CUresult (*)(CUstream, CUgreenCtx *);
+    using GreenResource = CUresult (*)(CUgreenCtx, CUdevResource *, CUdevResourceType);
+    static const auto entry = [](const char *name) -> void * {
+        void *p = nullptr;
+        cudaDriverEntryPointQueryResult q{};
+        if (cudaGetDriverEntryPointByVersion(name, &p, 12040, cudaEnableDefault, &q) != cudaSuccess ||
+            q != cudaDriverEntryPointSuccess) {
+            cudaGetLastError();
+            p = nullptr;
+        }
+        return p;
+    };
+    static const auto stream_green = reinterpret_cast<StreamGreen>(entry("cuStreamGetGreenCtx"));
+    static const auto green_resource = reinterpret_cast<GreenResource>(entry("cuGreenCtxGetDevResource"));
+    CUgreenCtx g = nullptr;
+    CUdevResource r{};
+    if (!h->stream || !stream_green || !green_resource || stream_green(h->stream, &g) != CUDA_SUCCESS || !g ||
+        green_resource(g, &r, CU_DEV_RESOURCE_TYPE_SM) != CUDA_SUCCESS)
+        return h->num_sms;
+    return std::min(h->num_sms, (int)r.sm.smCount);
+}
+
 LinePlan line_plan(const fdtd_plasma *h)
 {
     // a row weighs its nodes: an FP64 row is bound by the FP64 pipe, and the cells of a range cost next to nothing
-    return line1d_plan(h->nz, h->h_cells, h->num_sms, h->has_plasma ? (double)h->pitch : 0.0);
+    return line1d_plan(h->nz, h->h_cells, stream_sms(h), h->has_plasma ? (double)h->pitch : 0.0);
 }
 
 // whether the 1-D stepping kernel steps the grid, decided from sizes alone on first use
@@ -920,17 +946,23 @@ cudaError_t line_launch(fdtd_plasma *h, int nsteps)
     return launch_line1d<T>(h->stream, a, line_dtype(h), h->line_ctas);
 }
 
-int line_step(fdtd_plasma *h, int64_t nsteps)
+// up to nsteps steps; returns those left over when a launch is refused (CTAs that cannot all be resident, whatever
+// limits the process): nothing of it ran, and the step graphs take them and every later one
+int64_t line_step(fdtd_plasma *h, int64_t nsteps)
 {
-    for (int64_t left = nsteps; left > 0;) {
-        const int n = (int)std::min<int64_t>(left, 65536);
+    while (nsteps > 0) {
+        const int n = (int)std::min<int64_t>(nsteps, 65536);
         const cudaError_t e = h->g.precision == FDTD_F64 ? line_launch<double>(h, n) : line_launch<float>(h, n);
-        if (e != cudaSuccess) return cuda_fail(h, e, "1-D stepping kernel");
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            h->line_state = -1;
+            break;
+        }
         h->line_seq += (uint32_t)n;
         h->steps_done += n;
-        left -= n;
+        nsteps -= n;
     }
-    return FDTD_OK;
+    return nsteps;
 }
 
 int capture(fdtd_plasma *h, int nsteps, cudaGraphExec_t *out)
@@ -1553,7 +1585,8 @@ int fdtd_plasma_step(fdtd_plasma_t h, int64_t nsteps)
             const int rc = line_prepare(h);
             if (rc != FDTD_OK) return rc;
         }
-        if (h->line_state > 0) return line_step(h, nsteps);
+        if (h->line_state > 0) nsteps = line_step(h, nsteps);
+        if (nsteps == 0) return FDTD_OK;
     }
     if (!h->graphs_valid) {
         ensure_second_set(h);

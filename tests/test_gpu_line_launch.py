@@ -1,4 +1,7 @@
-"""The 1-D cooperative launch where it is refused or held up: while the caller's stream captures."""
+"""The 1-D cooperative launch where it is refused or held up: while the caller's stream captures, and on a stream
+that may use some of the SMs only."""
+import ctypes
+
 import numpy as np
 import pytest
 
@@ -50,3 +53,59 @@ def test_step_while_the_stream_captures(before):
         for s in (a, b):
             s.step(40)
         assert _same(a, b)
+
+
+class _GreenStream:
+    """A stream of a green context of at least `sms` SMs (driver API; no other process or stream is affected)."""
+
+    def __init__(self, sms):
+        import torch
+        torch.zeros(1, device="cuda")
+        try:
+            self.cu = ctypes.CDLL("libcuda.so.1")
+            for f in ("cuDeviceGetDevResource", "cuDevSmResourceSplitByCount", "cuDevResourceGenerateDesc",
+                      "cuGreenCtxCreate", "cuGreenCtxStreamCreate", "cuStreamDestroy_v2", "cuGreenCtxDestroy"):
+                getattr(self.cu, f)
+        except (OSError, AttributeError) as e:
+            pytest.skip(f"no green contexts here: {e}")
+        res = lambda: ctypes.create_string_buffer(144)   # CUdevResource: type, 92 bytes, 48 bytes
+        all_sms, part, rest, n = res(), res(), res(), ctypes.c_uint(1)
+        desc, self.ctx, self.ptr = ctypes.c_void_p(), ctypes.c_void_p(), ctypes.c_void_p()
+        self._call("cuDeviceGetDevResource", 0, all_sms, 1)
+        self._call("cuDevSmResourceSplitByCount", part, ctypes.byref(n), all_sms, rest, 0, sms)
+        self._call("cuDevResourceGenerateDesc", ctypes.byref(desc), part, 1)
+        self._call("cuGreenCtxCreate", ctypes.byref(self.ctx), desc, 0, 1)
+        self._call("cuGreenCtxStreamCreate", ctypes.byref(self.ptr), self.ctx, 1, 0)
+        self.sms = int(np.frombuffer(part.raw[96:100], dtype=np.uint32)[0])
+        self.stream = torch.cuda.ExternalStream(self.ptr.value)
+
+    def _call(self, name, *args):
+        rc = getattr(self.cu, name)(*args)
+        if rc:
+            pytest.skip(f"{name}: error {rc}")
+
+    def close(self):
+        self.stream.synchronize()
+        self._call("cuStreamDestroy_v2", self.ptr)
+        self._call("cuGreenCtxDestroy", self.ctx)
+
+
+@pytest.mark.parametrize("nv,coop", [(64, True), (512, False)])
+def test_stream_with_some_of_the_sms(nv, coop):
+    """A line whose state fits 16 SMs runs there, one that needs the whole device takes the step graphs; the results
+    are those of an ordinary stream."""
+    import torch
+    from paper_2211_05647_gb300 import Solver
+    sp = _spec(nz=3000, slab=(500, 2900), nv=nv)
+    b = Solver.from_spec(sp)
+    assert b.launch_shapes()["block_x"] > 0
+    g = _GreenStream(16)
+    assert 16 <= g.sms < torch.cuda.get_device_properties(0).multi_processor_count
+    a = Solver.from_spec(sp, stream=g.stream)
+    assert (a.launch_shapes()["block_x"] > 0) == coop
+    for n in (1, 70):
+        a.step(n)
+        b.step(n)
+    assert _same(a, b)
+    a.close()
+    g.close()
