@@ -249,7 +249,8 @@ int fdtd_plasma_check_canaries(fdtd_plasma_t h, int64_t *corrupted);
  * their plane loads, the bulk-copy ring for its chunks and the 1-D stepping kernel
  * for its neighbours' edges with an iteration or wall-clock limit, after which they
  * set an error word (reported as FDTD_ERR_TIMEOUT by fdtd_plasma_diagnostics
- * and by host reads of fdtd_plasma_read_fields) and return instead of hanging.  This launches one
+ * and by host reads of fdtd_plasma_read_fields, not by device reads; the
+ * state is void then, until fdtd_plasma_reset) and return instead of hanging.  This launches one
  * CTA that waits, with the same helper, on a barrier nothing arrives at, for
  * max_iter tries (1..2^20), and stores 1 in *gave_up (host) when the wait gave
  * up as designed, 0 if it completed.  Synchronous, on the legacy stream. */
@@ -261,6 +262,10 @@ int fdtd_selftest_wait_timeout(uint32_t max_iter, int32_t *gave_up);
  * passed on the GPU's global timer, then stores 1 in *gave_up (host).
  * Synchronous, on the legacy stream; FDTD_ERR_INVAL for a bad argument. */
 int fdtd_selftest_timed_wait(uint32_t limit_us, int32_t *gave_up);
+
+/* The same for the 1-D stepping kernel's wait for a neighbour's message (1 s
+ * there): one thread polls a box that nothing is sent to. */
+int fdtd_selftest_line_wait(uint32_t limit_us, int32_t *gave_up);
 
 /* Runtime options.  Without any, and without autotuned or cached shapes, the
  * sizes choose: 2-D FP32 whole grids of 6 M cells and more (nx a multiple of

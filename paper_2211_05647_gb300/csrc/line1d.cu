@@ -56,9 +56,11 @@ __device__ __forceinline__ void mail_put(uint64_t *box, T v, uint32_t tag)
     }
 }
 
-// wait for the message tagged `tag`; false if it did not come in time
+// wait for the message tagged `tag`; false if it did not come in time.  The neighbour runs: a cooperative grid
+// starts when all of its CTAs can be resident, and none of them before (beside a launch of another stream that
+// held 32 SMs for 3.6 s, all 152 started at its end), so it answers within microseconds.
 template <typename T>
-__device__ __forceinline__ bool mail_get(const uint64_t *box, T &v, uint32_t tag)
+__device__ __forceinline__ bool mail_get(const uint64_t *box, T &v, uint32_t tag, uint64_t limit_ns = kLineWaitNs)
 {
     uint64_t t0 = 0;
     for (uint32_t it = 1;; ++it) {
@@ -80,7 +82,7 @@ __device__ __forceinline__ bool mail_get(const uint64_t *box, T &v, uint32_t tag
         if ((it & 127u) == 0) {
             const uint64_t t = globaltimer_ns();
             if (!t0) t0 = t;
-            else if (t - t0 > kLineWaitNs) return false;
+            else if (t - t0 > limit_ns) return false;
         }
     }
 }
@@ -327,6 +329,13 @@ cudaError_t launch_line1d<double>(cudaStream_t st, const LineArgs<double> &a, in
     return dispatch_line<double, double>(st, a, ctas);
 }
 
+// one thread waits for a message that never comes
+__global__ void k_line_wait_selftest(const uint64_t *box, uint64_t limit_ns, int *gave_up)
+{
+    float v = 0.0f;
+    *gave_up = mail_get<float>(box, v, 1u, limit_ns) ? 0 : 1;
+}
+
 size_t line1d_smem_bytes(int f_dtype, int pitch, int rows, int nodes)
 {
     if (f_dtype == FDTD_DF_F64) return LineSmem<double, double>(pitch, rows, nodes).total;
@@ -335,3 +344,25 @@ size_t line1d_smem_bytes(int f_dtype, int pitch, int rows, int nodes)
 }
 
 }  // namespace fp
+
+using namespace fp;
+
+extern "C" int fdtd_selftest_line_wait(uint32_t limit_us, int32_t *gave_up)
+{
+    if (!gave_up || limit_us == 0 || limit_us > 1000000u)
+        return fp_set_global_error(FDTD_ERR_INVAL, "fdtd_selftest_line_wait: gave_up NULL or limit_us not in 1..10^6");
+    uint64_t *d = nullptr;   // the message box and the result
+    if (cudaMalloc(&d, 2 * sizeof(uint64_t)) != cudaSuccess)
+        return fp_set_global_error(FDTD_ERR_NOMEM, "cudaMalloc failed");
+    int h = -1;
+    cudaError_t e = cudaMemset(d, 0, 2 * sizeof(uint64_t));
+    if (e == cudaSuccess) {
+        k_line_wait_selftest<<<1, 1>>>(d, (uint64_t)limit_us * 1000u, reinterpret_cast<int *>(d + 1));
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaMemcpy(&h, d + 1, sizeof(int), cudaMemcpyDeviceToHost);
+    cudaFree(d);
+    if (e != cudaSuccess) return fp_set_global_error(FDTD_ERR_CUDA, cudaGetErrorString(e));
+    *gave_up = h;
+    return FDTD_OK;
+}

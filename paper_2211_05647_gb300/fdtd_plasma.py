@@ -154,6 +154,7 @@ SIGNATURES = {
     "fdtd_plasma_check_canaries": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(ctypes.c_int64)]),
     "fdtd_selftest_wait_timeout": (ctypes.c_int, [ctypes.c_uint32, ctypes.POINTER(ctypes.c_int32)]),
     "fdtd_selftest_timed_wait": (ctypes.c_int, [ctypes.c_uint32, ctypes.POINTER(ctypes.c_int32)]),
+    "fdtd_selftest_line_wait": (ctypes.c_int, [ctypes.c_uint32, ctypes.POINTER(ctypes.c_int32)]),
     "fdtd_plasma_set_option": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int, ctypes.c_int64]),
     "fdtd_plasma_launch_shapes": (ctypes.c_int, [ctypes.c_void_p, ctypes.POINTER(fdtd_tune_result)]),
     "fdtd_plasma_set_ports": (ctypes.c_int, [ctypes.c_void_p, ctypes.c_int32, ctypes.POINTER(ctypes.c_int64),
@@ -332,6 +333,14 @@ def selftest_timed_wait(limit_us: int = 2000) -> bool:
     lib = load_library()
     out = ctypes.c_int32(-1)
     _check(lib, None, lib.fdtd_selftest_timed_wait(int(limit_us), ctypes.byref(out)))
+    return out.value == 1
+
+
+def selftest_line_wait(limit_us: int = 2000) -> bool:
+    """Run the self-test of the 1-D stepping kernel's message wait; True when it gave up as designed."""
+    lib = load_library()
+    out = ctypes.c_int32(-1)
+    _check(lib, None, lib.fdtd_selftest_line_wait(int(limit_us), ctypes.byref(out)))
     return out.value == 1
 
 

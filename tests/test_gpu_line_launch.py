@@ -1,5 +1,5 @@
 """The 1-D cooperative launch where it is refused or held up: while the caller's stream captures, and on a stream
-that may use some of the SMs only."""
+that may use some of the SMs only; and the bounded wait of its CTAs."""
 import ctypes
 
 import numpy as np
@@ -16,6 +16,17 @@ def _spec(nz=2000, slab=(900, 1400), nv=64, seed=3):
     return sp
 
 
+def _make(sp, stream=None):
+    """A solver whose plasma is driven from the first step."""
+    from paper_2211_05647_gb300 import Solver
+    s = Solver.from_spec(sp, stream=stream)
+    rng = np.random.default_rng(4)
+    nz = sp["grid"]["nz"]
+    s.write("ex", rng.standard_normal(nz + 1))
+    s.write("hy", rng.standard_normal(nz) / 377.0)
+    return s
+
+
 def _state(s):
     return {q: s.read(q, device=False).copy() for q in ("ex", "hy", "j", "df")}
 
@@ -30,10 +41,10 @@ def test_step_while_the_stream_captures(before):
     """Refused with an error that leaves the capture and the handle as they were: the first step of a handle as any
     later one, and the handle still takes the cooperative kernel afterwards."""
     import torch
-    from paper_2211_05647_gb300 import FdtdError, Solver
+    from paper_2211_05647_gb300 import FdtdError
     st = torch.cuda.Stream()
     with torch.cuda.stream(st):
-        a, b = Solver.from_spec(_spec(), stream=st), Solver.from_spec(_spec(), stream=st)
+        a, b = _make(_spec(), st), _make(_spec(), st)
         if before:
             a.step(before)
             b.step(before)
@@ -95,13 +106,12 @@ def test_stream_with_some_of_the_sms(nv, coop):
     """A line whose state fits 16 SMs runs there, one that needs the whole device takes the step graphs; the results
     are those of an ordinary stream."""
     import torch
-    from paper_2211_05647_gb300 import Solver
     sp = _spec(nz=3000, slab=(500, 2900), nv=nv)
-    b = Solver.from_spec(sp)
+    b = _make(sp)
     assert b.launch_shapes()["block_x"] > 0
     g = _GreenStream(16)
     assert 16 <= g.sms < torch.cuda.get_device_properties(0).multi_processor_count
-    a = Solver.from_spec(sp, stream=g.stream)
+    a = _make(sp, g.stream)
     assert (a.launch_shapes()["block_x"] > 0) == coop
     for n in (1, 70):
         a.step(n)
@@ -109,3 +119,19 @@ def test_stream_with_some_of_the_sms(nv, coop):
     assert _same(a, b)
     a.close()
     g.close()
+
+
+def test_wait_gives_up_after_its_limit():
+    """A message that never comes is given up on after the limit, not sooner and not never."""
+    import time
+    from paper_2211_05647_gb300 import FdtdError, Solver, selftest_line_wait
+    selftest_line_wait(10)                        # load and warm the module
+    t0 = time.perf_counter()
+    assert selftest_line_wait(2000) is True
+    assert 2e-3 <= time.perf_counter() - t0 < 1.0
+    for bad in (0, 10 ** 7):
+        with pytest.raises(FdtdError):
+            selftest_line_wait(bad)
+    s = Solver.from_spec(_spec())
+    s.step(20)
+    assert s.diagnostics()["finite"]
