@@ -411,6 +411,7 @@ struct fdtd_batch {
     int64_t max_steps;   // steps a launch: the source table's length, at most 1024 and 16 MB (32 steps for any batch)
     int64_t steps_done;
     std::map<int64_t, cudaGraphExec_t> graphs;
+    CopyHome home;
     std::string err;
     cudaError_t (*launch)(fdtd_batch *, cudaStream_t, int);
     // row-shape candidates (vectors per lane, lanes per row) for this row length; [0] is the default
@@ -645,6 +646,9 @@ int fdtd_batch_create(const fdtd_run_desc *runs, int32_t nruns, const fdtd_runti
         destroy_batch(b);
         return code;
     };
+    if (cudaGetDevice(&b->home.dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&b->home.sms, cudaDevAttrMultiProcessorCount, b->home.dev) != cudaSuccess)
+        return bail(FDTD_ERR_CUDA, "device setup failed");
     if (cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking) != cudaSuccess)
         return bail(FDTD_ERR_CUDA, "stream creation failed");
     b->precision = g0.precision;
@@ -929,12 +933,12 @@ int fdtd_batch_read(fdtd_batch_t b, int32_t run, int which, void *dst, size_t by
     cudaError_t e;
     if (which == FDTD_DF) {
         const size_t row = (size_t)b->nnode * b->df_esz, dp = (size_t)b->pitch * b->df_esz;
-        e = copy_rows(b->stream, dst, (char *)b->df + b->row_off[run] * dp, b->nslot[run], row, dp, kind, true);
+        e = copy_rows(b->stream, dst, (char *)b->df + b->row_off[run] * dp, b->nslot[run], row, dp, kind, true, b->home);
     } else {
         char *src = which == FDTD_EX   ? (char *)b->E + b->e_off[run] * b->esz
                           : which == FDTD_HY ? (char *)b->H + b->h_off[run] * b->esz
                                              : (char *)b->jslot + b->row_off[run] * b->esz;
-        e = copy_linear(b->stream, dst, src, bytes, kind, true);
+        e = copy_linear(b->stream, dst, src, bytes, kind, true, b->home);
     }
     if (e == cudaSuccess && !dst_is_device) e = cudaStreamSynchronize(b->stream);
     if (e != cudaSuccess) return bfail(b, FDTD_ERR_CUDA, "read: %s", cudaGetErrorString(e));

@@ -874,9 +874,8 @@ bool line_steps(fdtd_plasma *h)
         const int f_dtype = line_dtype(h), pitch = h->has_plasma ? h->pitch : 0;
         if (pitch / (f_dtype == FDTD_DF_BF16 ? 8 : (f_dtype == FDTD_DF_F64 ? 2 : 4)) > 128) return false;
         const LinePlan p = line_plan(h);
-        int dev = 0, most = 0;
-        if (cudaGetDevice(&dev) != cudaSuccess ||
-            cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess) {
+        int most = 0;
+        if (cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->dev) != cudaSuccess) {
             cudaGetLastError();
             return false;
         }
@@ -1079,6 +1078,7 @@ int create_impl(const fdtd_grid_desc *g, const fdtd_runtime_desc *rt, fdtd_plasm
     h->esz = g->precision == FDTD_F64 ? 8 : 4;
     int dev = 0;
     cudaError_t ce = cudaGetDevice(&dev);
+    h->dev = dev;
     if (ce == cudaSuccess) ce = cudaDeviceGetAttribute(&h->num_sms, cudaDevAttrMultiProcessorCount, dev);
     if (ce == cudaSuccess) ce = cudaStreamCreateWithFlags(&h->cap, cudaStreamNonBlocking);
     if (ce != cudaSuccess) {
@@ -1575,6 +1575,7 @@ int fdtd_plasma_step(fdtd_plasma_t h, int64_t nsteps)
         return fail(h, FDTD_ERR_STATE, "a sub-domain with neighbours steps by fdtd_plasma_step_half, exchanging halos");
     if (nsteps == 0) return FDTD_OK;
     if (line_steps(h)) {
+        const DeviceGuard guard(h->dev);   // (a graph launch needs none)
         // the launch carries the step and message counters as arguments: it is not for replay in a caller's graph
         // (the step graphs cannot be captured either).  Asked before anything is put on the stream.
         cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
@@ -2113,10 +2114,10 @@ static int copy_quantity(fdtd_plasma_t h, int which, void *host_or_dev, size_t b
     if (which == FDTD_DF || which == FDTD_F0) {
         void *rows = which == FDTD_DF ? h->df : h->g0;
         const size_t row = (size_t)h->nnode * h->df_esz, dpitch = (size_t)h->pitch * h->df_esz;
-        CK(h, copy_rows(h->stream, host_or_dev, rows, h->nkin, row, dpitch, kind, out));
+        CK(h, copy_rows(h->stream, host_or_dev, rows, h->nkin, row, dpitch, kind, out, {h->dev, h->num_sms}));
     } else {
         void *dev = which == FDTD_J ? h->jslot : h->f[which];
-        CK(h, copy_linear(h->stream, host_or_dev, dev, bytes, kind, out));
+        CK(h, copy_linear(h->stream, host_or_dev, dev, bytes, kind, out, {h->dev, h->num_sms}));
     }
     if (!is_device) {
         int errw = 0;

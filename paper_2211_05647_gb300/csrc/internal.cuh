@@ -9,6 +9,7 @@
 #include <string>
 #include <vector>
 
+#include "copy_route.cuh"
 #include "fdtd_plasma.h"
 
 namespace fp {
@@ -286,13 +287,30 @@ cudaError_t launch_compact_scatter(cudaStream_t st, const double *d, const Compa
 // dst[i] = (float)src[i], i < n (round to nearest, as the host conversion)
 cudaError_t launch_to_f32(cudaStream_t st, const double *src, float *dst, int64_t n);
 
+// makes a device current for a scope: what a call launches goes to the device its handle was made on
+struct DeviceGuard {
+    int was = -1;
+    explicit DeviceGuard(int dev)
+    {
+        int now = dev;
+        if (cudaGetDevice(&now) == cudaSuccess && now != dev && cudaSetDevice(dev) == cudaSuccess) was = now;
+    }
+    ~DeviceGuard()
+    {
+        if (was >= 0) cudaSetDevice(was);
+    }
+    DeviceGuard(const DeviceGuard &) = delete;
+    DeviceGuard &operator=(const DeviceGuard &) = delete;
+};
+
 // bytes between one of the solver's arrays and the caller's memory (out: to the caller), stream-ordered; kind says
 // where the caller's memory is (rows.cu)
-cudaError_t copy_linear(cudaStream_t st, void *theirs, void *ours, size_t bytes, cudaMemcpyKind kind, bool out);
+cudaError_t copy_linear(cudaStream_t st, void *theirs, void *ours, size_t bytes, cudaMemcpyKind kind, bool out,
+                        const CopyHome &home);
 // delta-f rows between the padded layout (pitch bytes apart) and the packed one of read / write_fields; out:
 // padded -> packed.  kind says where the packed side is (rows.cu)
 cudaError_t copy_rows(cudaStream_t st, void *packed, void *padded, int64_t rows, size_t row, size_t pitch,
-                      cudaMemcpyKind kind, bool out);
+                      cudaMemcpyKind kind, bool out, const CopyHome &home);
 
 // delta-f row pitch (elements) for nnode nodes of the given storage type
 int kinetic_pitch(int nnode, int f_dtype);
@@ -408,7 +426,7 @@ struct fdtd_plasma {
     fdtd_runtime_desc rt;
     cudaStream_t stream;      // caller's stream
     cudaStream_t cap;         // private stream used for graph capture
-    int num_sms;
+    int num_sms, dev;
     double dt;
     int64_t nx, ny, nz;
     size_t esz;               // field element size

@@ -65,27 +65,27 @@ __global__ void __launch_bounds__(256) k_copy(U *__restrict__ dst, const U *__re
 }
 
 template <typename U>
-cudaError_t run_copy(cudaStream_t st, void *dst, const void *src, size_t bytes)
+cudaError_t run_copy(cudaStream_t st, void *dst, const void *src, size_t bytes, const CopyHome &home)
 {
     const uint32_t n = (uint32_t)(bytes / sizeof(U));
-    const uint32_t blocks = std::min<uint32_t>((n + 256 * kRowsUnroll - 1) / (256 * kRowsUnroll), 152 * 8);
-    return launch_pdl(k_copy<U>, dim3(blocks), dim3(256), 0, st, static_cast<U *>(dst), static_cast<const U *>(src), n);
+    const DeviceGuard guard(home.dev);
+    return launch_pdl(k_copy<U>, dim3(copy_blocks(n, 256 * kRowsUnroll, home)), dim3(256), 0, st, static_cast<U *>(dst), static_cast<const U *>(src), n);
 }
 
-// whether kernels of the current device may read and write the caller's memory (a copy engine reaches other places)
-bool on_this_device(const void *p)
+bool reaches(const void *p, const CopyHome &home)
 {
-    int dev = 0;
     cudaPointerAttributes at{};
-    if (cudaGetDevice(&dev) == cudaSuccess && cudaPointerGetAttributes(&at, p) == cudaSuccess)
-        return at.type == cudaMemoryTypeDevice && at.device == dev;
+    if (cudaPointerGetAttributes(&at, p) == cudaSuccess)
+        return kernel_reaches(at.type == cudaMemoryTypeDevice, at.device, home);
     cudaGetLastError();
     return false;
 }
 
 template <typename U>
-cudaError_t run(cudaStream_t st, void *dst, const void *src, int64_t rows, size_t row, size_t pitch, bool pack)
+cudaError_t run(cudaStream_t st, void *dst, const void *src, int64_t rows, size_t row, size_t pitch, bool pack,
+                const CopyHome &home)
 {
+    const DeviceGuard guard(home.dev);
     const uint32_t per = (uint32_t)(row / sizeof(U)), n = (uint32_t)(rows * per);
     // i / per = (i * mul) >> shift for every i < 2^31: mul = ceil(2^(31 + k) / per), 2^k >= per
     int k = 0;
@@ -101,7 +101,8 @@ cudaError_t run(cudaStream_t st, void *dst, const void *src, int64_t rows, size_
 
 }  // namespace
 
-cudaError_t copy_linear(cudaStream_t st, void *theirs, void *ours, size_t bytes, cudaMemcpyKind kind, bool out)
+cudaError_t copy_linear(cudaStream_t st, void *theirs, void *ours, size_t bytes, cudaMemcpyKind kind, bool out,
+                        const CopyHome &home)
 {
     void *dst = out ? theirs : ours;
     const void *src = out ? ours : theirs;
@@ -109,35 +110,35 @@ cudaError_t copy_linear(cudaStream_t st, void *theirs, void *ours, size_t bytes,
     // smallest keep the plain copy: a call with the pointer's check and a launch is a microsecond longer on the
     // host, which bounds a program that reads a few kilobytes after every step (39 against 43 us a step and four
     // reads)
-    if (kind == cudaMemcpyDeviceToDevice && bytes > 16384 && bytes <= (size_t)16 << 20 && on_this_device(theirs)) {
+    if (kind == cudaMemcpyDeviceToDevice && bytes > 16384 && bytes <= (size_t)16 << 20 && reaches(theirs, home)) {
         size_t u = 16;
         while (u > 2 && (((uintptr_t)dst | (uintptr_t)src | bytes) & (u - 1))) u >>= 1;
         switch (u) {
-        case 16: return run_copy<uint4>(st, dst, src, bytes);
-        case 8: return run_copy<uint2>(st, dst, src, bytes);
-        case 4: return run_copy<uint32_t>(st, dst, src, bytes);
+        case 16: return run_copy<uint4>(st, dst, src, bytes, home);
+        case 8: return run_copy<uint2>(st, dst, src, bytes, home);
+        case 4: return run_copy<uint32_t>(st, dst, src, bytes, home);
         default:
-            if (!(((uintptr_t)dst | (uintptr_t)src | bytes) & 1)) return run_copy<uint16_t>(st, dst, src, bytes);
+            if (!(((uintptr_t)dst | (uintptr_t)src | bytes) & 1)) return run_copy<uint16_t>(st, dst, src, bytes, home);
         }
     }
     return cudaMemcpyAsync(dst, src, bytes, kind, st);
 }
 
 cudaError_t copy_rows(cudaStream_t st, void *packed, void *padded, int64_t rows, size_t row, size_t pitch,
-                      cudaMemcpyKind kind, bool out)
+                      cudaMemcpyKind kind, bool out, const CopyHome &home)
 {
     void *dst = out ? packed : padded;
     const void *src = out ? padded : packed;
-    if (row == pitch) return copy_linear(st, packed, padded, (size_t)rows * row, kind, out);
+    if (row == pitch) return copy_linear(st, packed, padded, (size_t)rows * row, kind, out, home);
     size_t u = 16;
     while (u > 1 && (row % u || pitch % u || (uintptr_t)packed % u)) u >>= 1;
     if (kind == cudaMemcpyDeviceToDevice && rows > 0 && u >= 2 && (uint64_t)rows * (row / u) < ((uint64_t)1 << 31) &&
-        on_this_device(packed)) {
+        reaches(packed, home)) {
         switch (u) {
-        case 16: return run<uint4>(st, dst, src, rows, row, pitch, out);
-        case 8: return run<uint2>(st, dst, src, rows, row, pitch, out);
-        case 4: return run<uint32_t>(st, dst, src, rows, row, pitch, out);
-        default: return run<uint16_t>(st, dst, src, rows, row, pitch, out);
+        case 16: return run<uint4>(st, dst, src, rows, row, pitch, out, home);
+        case 8: return run<uint2>(st, dst, src, rows, row, pitch, out, home);
+        case 4: return run<uint32_t>(st, dst, src, rows, row, pitch, out, home);
+        default: return run<uint16_t>(st, dst, src, rows, row, pitch, out, home);
         }
     }
     return out ? cudaMemcpy2DAsync(packed, row, padded, pitch, row, rows, kind, st)
