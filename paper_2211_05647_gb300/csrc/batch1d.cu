@@ -159,15 +159,17 @@ __host__ __device__ constexpr size_t batch_smem_bytes(int pitch)
 
 // CTAs per SM the registers are budgeted for: three with FP32 rows (80 registers, no spill: 0.316 -> 0.288 ms a
 // step on the 256-run workload), two otherwise (BF16 rows lost at three: 0.189 -> 0.213 ms, the packing then
-// taking clusters of eight)
-template <typename TS>
+// taking clusters of eight; the longest FP32 rows hold eight vectors a lane, twice: 40 bytes of spills at 128
+// registers, and still ahead of four at three CTAs -- 128 runs, rows of 256 nodes 82.8 -> 73.1 us a step, of 512
+// 102.6 -> 86.0)
+template <typename TS, int VPL>
 constexpr int batch_min_blocks()
 {
-    return std::is_same<TS, float>::value ? 3 : 2;
+    return std::is_same<TS, float>::value && VPL < 8 ? 3 : 2;
 }
 
 template <typename TS, typename T, int VPL, int L>
-__global__ void __launch_bounds__(kBatchThreads, batch_min_blocks<TS>()) k_batch1d(BatchArgs<T> a)
+__global__ void __launch_bounds__(kBatchThreads, batch_min_blocks<TS, VPL>()) k_batch1d(BatchArgs<T> a)
 {
     cg::cluster_group cluster = cg::this_cluster();
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -528,9 +530,9 @@ int max_clusters(int ctas)
 }
 
 // Row-shape candidates (storage, precision, vectors per row): the first is the built-in choice and
-// fixes the cluster packing; fdtd_batch_autotune may switch to another (two vectors a lane, twice the
-// lanes: eight vectors a lane spill at the kernel's 128 registers).  The FP64 validation instantiation
-// keeps the built-in shape only.
+// fixes the cluster packing; fdtd_batch_autotune may switch to another.  The built-in one sums J in the order of the
+// single-run default (kinetic_default_shape), so that a run of a batch has the bits it has alone.  The FP64 validation
+// instantiation keeps the built-in shape only.
 template <typename TS, typename T, int VPL, int L>
 fdtd_batch::Shape shape_of()
 {
@@ -541,7 +543,7 @@ template <typename TS, typename T>
 bool pick(int V, std::vector<fdtd_batch::Shape> &sh, int (**maxc)(int))
 {
     sh.clear();
-    constexpr bool more = !std::is_same<T, double>::value;
+    constexpr bool more = !std::is_same<T, double>::value, f32 = std::is_same<TS, float>::value;
     switch (V) {
     case 1: sh = {shape_of<TS, T, 1, 1>()}; *maxc = max_clusters<TS, T, 1, 1>; break;
     case 2:
@@ -555,9 +557,14 @@ bool pick(int V, std::vector<fdtd_batch::Shape> &sh, int (**maxc)(int))
         *maxc = max_clusters<TS, T, 4, 1>;
         break;
     case 8:
-        sh = {shape_of<TS, T, 4, 2>()};
-        if constexpr (more) sh.push_back(shape_of<TS, T, 2, 4>());
-        *maxc = max_clusters<TS, T, 4, 2>;
+        if constexpr (f32) {
+            sh = {shape_of<TS, T, 2, 4>(), shape_of<TS, T, 4, 2>()};
+            *maxc = max_clusters<TS, T, 2, 4>;
+        } else {
+            sh = {shape_of<TS, T, 4, 2>()};
+            if constexpr (more) sh.push_back(shape_of<TS, T, 2, 4>());
+            *maxc = max_clusters<TS, T, 4, 2>;
+        }
         break;
     case 16:
         sh = {shape_of<TS, T, 4, 4>()};
@@ -570,13 +577,23 @@ bool pick(int V, std::vector<fdtd_batch::Shape> &sh, int (**maxc)(int))
         *maxc = max_clusters<TS, T, 4, 8>;
         break;
     case 64:
-        sh = {shape_of<TS, T, 4, 16>()};
-        if constexpr (more) sh.push_back(shape_of<TS, T, 2, 32>());
-        *maxc = max_clusters<TS, T, 4, 16>;
+        if constexpr (f32) {
+            sh = {shape_of<TS, T, 8, 8>(), shape_of<TS, T, 4, 16>()};
+            *maxc = max_clusters<TS, T, 8, 8>;
+        } else {
+            sh = {shape_of<TS, T, 4, 16>()};
+            if constexpr (more) sh.push_back(shape_of<TS, T, 2, 32>());
+            *maxc = max_clusters<TS, T, 4, 16>;
+        }
         break;
     case 128:
-        sh = {shape_of<TS, T, 4, 32>()};
-        *maxc = max_clusters<TS, T, 4, 32>;
+        if constexpr (f32) {
+            sh = {shape_of<TS, T, 8, 16>(), shape_of<TS, T, 4, 32>()};
+            *maxc = max_clusters<TS, T, 8, 16>;
+        } else {
+            sh = {shape_of<TS, T, 4, 32>()};
+            *maxc = max_clusters<TS, T, 4, 32>;
+        }
         break;
     default: return false;
     }
