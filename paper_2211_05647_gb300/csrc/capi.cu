@@ -605,7 +605,8 @@ cudaError_t part_mid(fdtd_plasma *h, cudaStream_t st, int kstep, const FieldSet<
             const double vth = std::sqrt(kQe * h->pl.te_ev / kMe);
             const double dvpar = 2.0 * h->pl.vmax_vth * vth / h->pl.nv;
             const int nperp = h->pl.vgrid == FDTD_VGRID_CART2D ? h->pl.nv_perp : 1;
-            e = launch_kinetic_nl<T>(st, a, h->pl.nv, nperp, dvpar, kQe / kMe, h->dt, h->num_sms);
+            e = launch_kinetic_nl<T>(st, a, h->pl.nv, nperp, dvpar, kQe / kMe, h->dt, h->num_sms,
+                                     h->sd_on ? h->rows_global : h->nkin);
         } else {
             const KinShape k = kin_shape(h);
             e = launch_kinetic<T>(st, a, h->pl.f_dtype, h->num_sms, k.vpl, k.l, k.bps, k.stages);
@@ -1399,7 +1400,7 @@ int fdtd_plasma_set_plasma(fdtd_plasma_t h, const fdtd_plasma_desc *p)
     // density: compact the plasma cells
     const int64_t np = pol_len(h);
     std::vector<double> dens(h->sd_on ? np : 0);
-    int64_t slot_base = 0;
+    int64_t slot_base = 0, rows_global = -1;
     if (h->sd_on) {
         // a sub-domain reads its planes of the global density array; its slots are numbered after the
         // global plasma slots below its first owned plane
@@ -1409,11 +1410,13 @@ int fdtd_plasma_set_plasma(fdtd_plasma_t h, const fdtd_plasma_desc *p)
         if (p->density_on_device) CK(h, cudaMemcpy(all.data(), p->density, npg * 8, cudaMemcpyDeviceToHost));
         else std::memcpy(all.data(), p->density, npg * 8);
         const int64_t first = (h->sd_origin + h->sd_lo) * plane;
-        for (int64_t c = 0; c < first; ++c) {
+        auto updated = [&](int64_t c) {
             const int64_t i = c % h->nx, j = (c / h->nx) % h->ny, k = c / plane;
-            const bool upd = h->sd_axis == 1 ? (i >= 1 && c / h->nx >= 1) : (j >= 1 && k >= 1);
-            if (all[c] > 0.0 && upd) ++slot_base;
-        }
+            return h->sd_axis == 1 ? (i >= 1 && c / h->nx >= 1) : (j >= 1 && k >= 1);
+        };
+        for (int64_t c = 0; c < first; ++c) slot_base += all[c] > 0.0 && updated(c);
+        rows_global = slot_base;
+        for (int64_t c = first; c < npg && p->nonlinear; ++c) rows_global += all[c] > 0.0 && updated(c);
         std::memcpy(dens.data(), all.data() + h->sd_origin * plane, np * 8);
         for (int64_t c = 0; c < np; ++c) {     // ghost planes carry no plasma
             const int64_t l = c / plane;
@@ -1524,6 +1527,7 @@ int fdtd_plasma_set_plasma(fdtd_plasma_t h, const fdtd_plasma_desc *p)
     }
     h->has_plasma = 1;
     h->slot_base = slot_base;
+    h->rows_global = rows_global;
     h->nkin = (int64_t)ns;
     h->kin_vpl = h->kin_l = h->kin_bps = h->kin_stages = h->kin_forced = 0;
     apply_cached_kinetic(h);

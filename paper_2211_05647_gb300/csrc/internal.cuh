@@ -339,7 +339,7 @@ template <typename T>
 cudaError_t launch_kinetic_f0(cudaStream_t st, const KinArgs<T> &a, const F0Args<T> &f, int num_sms);
 template <typename T>
 cudaError_t launch_kinetic_nl(cudaStream_t st, const KinArgs<T> &a, int npar, int nperp, double dvpar, double qm,
-                              double dt, int num_sms);
+                              double dt, int num_sms, int64_t rows_global);   // rows_global: the whole grid's rows
 
 struct DiagArgs {
     int ndim;
@@ -457,6 +457,7 @@ struct fdtd_plasma {
     int sd_on, sd_axis, sd_half;
     int64_t sd_nglobal, sd_origin, sd_extent, sd_lo, sd_hi;
     int64_t slot_base;        // global plasma-slot index of local slot 0
+    int64_t rows_global;      // plasma slots of the whole grid (sub-domains of the nonlinear update)
     // plasma
     int has_plasma;
     fdtd_plasma_desc pl;

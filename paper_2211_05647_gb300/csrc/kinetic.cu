@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(256) k_kinetic_nl(KinArgs<T> a, int npar, int 
     }
 }
 
-// Column walk, for rows whose v_perp columns are at least a 32-byte sector (nperp * sizeof(T) >= 32).
+// Column walk, for rows whose v_perp columns are at least a 32-byte sector (nl_walks below).
 // Every node needs only its v_par neighbours and its mirror, all of the same v_perp column: a lane owns C
 // adjacent columns (one 16-byte vector, or one value when nperp is not a multiple of the vector) and walks
 // them from both ends towards the middle, in pairs (a, npar - 1 - a).  The face flux a node shares with its
@@ -190,7 +190,8 @@ __global__ void __launch_bounds__(256) k_kinetic_nl(KinArgs<T> a, int npar, int 
 // nodes of a 512 x 512 grid with a radius-128 column) and by what 16 warps a SM keep in flight: the step of that
 // grid takes 0.100 ms against 0.265 ms with the staged rows below (measured with the plain loads and stores
 // 0.104; two-pair chunks at three CTAs a SM 0.104, four-pair chunks squeezed into three CTAs 0.139; two
-// columns a lane 0.104-0.131).
+// columns a lane 0.104-0.131).  FP64 keeps the same shape: 40 to 60 bytes of spills at the same 128 registers, and
+// bound by the FP64 pipe (20 k rows of 32 x 32 nodes: 1.93 ms a step staged, 0.75 walked).
 constexpr int kNlU = 4;
 
 template <typename T, int C>
@@ -345,15 +346,48 @@ cudaError_t run_kinetic_nl_walk(cudaStream_t st, const KinArgs<T> &a, int npar, 
     const int64_t rows = 8 * (32 / L);
     int64_t blocks = (a.nslots + rows - 1) / rows;
     blocks = std::min<int64_t>(blocks, (int64_t)num_sms * std::max(per_sm, 1));
+    // CTAs that start while the H stencil ends gather on the SMs it leaves first; the long FP64 rows, whose tables
+    // allow fewest of them a SM, then wait for one another's FP64 pipe (64 x 16 nodes, 441 rows: 298 us a step
+    // launched early, 157 so)
+    if (sizeof(T) == 8 && smem >= 24 * 1024)
+        return launch_plain(kern, dim3((unsigned)blocks), dim3(256), smem, st, a, npar, nperp, (T)(1.0 / dvpar), (T)qm,
+                            (T)dt);
     return launch_pdl(kern, dim3((unsigned)blocks), dim3(256), smem, st, a, npar, nperp, (T)(1.0 / dvpar), (T)qm, (T)dt);
+}
+
+// lanes a row of nperp columns, C a lane (single columns: nperp is not a multiple of a vector and at least 5)
+inline int nl_walk_lanes(int nperp, int C)
+{
+    int L = C == 1 ? 8 : 2;
+    while (L < 32 && L * C < nperp) L <<= 1;
+    return L;
+}
+
+// Whether rows of nperp columns are walked, in a grid of `rows` of them.  A column step has to be a whole 32-byte
+// sector: the walk reads and writes nothing but the rows then (0.100 against 0.265 ms a step, see above); of
+// narrower columns (the signed grid has one) it would use a part of each sector and move the rest in vain.  Where rows
+// are few, what counts is a lane's chain of nodes, a thirty-second of a row in the staged kernel:
+//  two lanes a row: from 32 rows a SM (us a step walked / staged -- FP64 32 x 4 nodes, 441 rows 81 / 56, 2453 82 / 72,
+//      5025 83 / 87; FP32 64 x 8, 441 rows 18.1 / 11.1, 5025 19.7 / 22.5);
+//  FP64, four or eight lanes: not below half a row a SM (32 x 8, 49 rows 71 / 37, 197 81 / 117), but for eight
+//      lanes with no more rows than give each sub-core of one SM a warp (32 x 16, 13 rows 45 / 65, 49 81 / 65).
+// Otherwise at any number (FP32 32 x 32: 13 rows 9.5 / 16.0).  The two round differently, so a sub-domain goes by the
+// whole grid's rows.
+inline bool nl_walks(int64_t rows, int nperp, bool f64, int num_sms)
+{
+    const int vec = f64 ? 2 : 4;
+    if (nperp * (f64 ? 8 : 4) < 32) return false;
+    const int L = nl_walk_lanes(nperp, nperp % vec ? 1 : vec);
+    if (L == 2) return rows >= 32 * (int64_t)num_sms;
+    if (f64 && L <= 8) return rows >= num_sms / 2 || (L == 8 && rows <= 16);
+    return true;
 }
 
 template <typename T, int C>
 cudaError_t dispatch_kinetic_nl_walk(cudaStream_t st, const KinArgs<T> &a, int npar, int nperp, double dvpar,
                                      double qm, double dt, int num_sms)
 {
-    int L = C == 1 ? 8 : 2;   // single columns: nperp is not a multiple of a vector and at least 5
-    while (L < 32 && L * C < nperp) L <<= 1;
+    const int L = nl_walk_lanes(nperp, C);
     if constexpr (C > 1) {
         if (L == 2) return run_kinetic_nl_walk<T, C, 2>(st, a, npar, nperp, dvpar, qm, dt, num_sms);
         if (L == 4) return run_kinetic_nl_walk<T, C, 4>(st, a, npar, nperp, dvpar, qm, dt, num_sms);
@@ -367,13 +401,10 @@ cudaError_t dispatch_kinetic_nl_walk(cudaStream_t st, const KinArgs<T> &a, int n
 
 template <typename T>
 cudaError_t launch_kinetic_nl(cudaStream_t st, const KinArgs<T> &a, int npar, int nperp, double dvpar, double qm,
-                              double dt, int num_sms)
+                              double dt, int num_sms, int64_t rows_global)
 {
     if (a.nslots == 0) return cudaSuccess;
-    // a column step of a whole 32-byte sector or more: the walk reads and writes nothing but the rows
-    // (0.100 against 0.265 ms a step, see above).  Narrower columns (the signed grid has one) would use a
-    // part of each sector and move the rest in vain: those rows are staged whole.
-    if ((size_t)nperp * sizeof(T) >= 32)
+    if (nl_walks(rows_global, nperp, sizeof(T) == 8, num_sms))
         return nperp % Vec<T>::n == 0
                    ? dispatch_kinetic_nl_walk<T, Vec<T>::n>(st, a, npar, nperp, dvpar, qm, dt, num_sms)
                    : dispatch_kinetic_nl_walk<T, 1>(st, a, npar, nperp, dvpar, qm, dt, num_sms);
@@ -393,9 +424,9 @@ cudaError_t launch_kinetic_nl(cudaStream_t st, const KinArgs<T> &a, int npar, in
 }
 
 template cudaError_t launch_kinetic_nl<float>(cudaStream_t, const KinArgs<float> &, int, int, double, double, double,
-                                              int);
+                                              int, int64_t);
 template cudaError_t launch_kinetic_nl<double>(cudaStream_t, const KinArgs<double> &, int, int, double, double,
-                                               double, int);
+                                               double, int, int64_t);
 
 // --------------------------------------------------------- evolving F0
 // Speed grid with an evolving isotropic part (the F0 equation of the two-term
