@@ -117,8 +117,10 @@ struct KinArgs {
     int store_j;               // k_kinetic: store J^{n+1/2} per slot (the last step of a sequence, or
                                // when something reads it every step); E is updated either way
     int *err;                  // set to 1 if a bounded wait of the bulk-copy ring kernel gave up
-    int after_stencil;         // k_kinetic: the launch before this one is a stencil of the same sequence (it may
-                               // then start, and read its first rows, while that stencil finishes)
+    int after_stencil;         // k_kinetic: what wrote delta f last has ended by the time this launch may start: within
+                               // a step sequence another launch, which waits before it lets this one start (pdl_enter),
+                               // lies between (an H update, an E history push); it then reads its first rows before
+                               // its own wait.  0: the second half of a split step, where a write may come between
 };
 
 // Isotropic-F0 evolution (speed grid): per-node tables, each `pitch` long,
