@@ -168,7 +168,8 @@ constexpr int batch_min_blocks()
     return std::is_same<TS, float>::value && VPL < 8 ? 3 : 2;
 }
 
-template <typename TS, typename T, int VPL, int L>
+// VS: vectors a partial sum (row_update_to)
+template <typename TS, typename T, int VPL, int L, int VS>
 __global__ void __launch_bounds__(kBatchThreads, batch_min_blocks<TS, VPL>()) k_batch1d(BatchArgs<T> a)
 {
     cg::cluster_group cluster = cg::this_cluster();
@@ -292,7 +293,7 @@ __global__ void __launch_bounds__(kBatchThreads, batch_min_blocks<TS, VPL>()) k_
                 V *rp = reinterpret_cast<V *>(a.df) + cur.grow * (a.pitch / VEC);
                 T sm = T(0), cm = T(0);
                 if (cur.valid)
-                    row_update<TS, T, VPL, L>(rp, cur.v, s_al, s_be, s_w, cur.dn * cur.e, l, (uint32_t)cur.grow, step,
+                    row_update<TS, T, VPL, L, VS>(rp, cur.v, s_al, s_be, s_w, cur.dn * cur.e, l, (uint32_t)cur.grow, step,
                                               key, sm, cm);
                 const T J = row_reduce<T, L>(sm, cm);
                 if (cur.valid && l == 0) {
@@ -454,7 +455,7 @@ void bfree(fdtd_batch *b, void *p)
     else cudaFree(p);
 }
 
-template <typename TS, typename T, int VPL, int L>
+template <typename TS, typename T, int VPL, int L, int VS>
 cudaError_t launch_t(fdtd_batch *b, cudaStream_t st, int nsteps)
 {
     BatchArgs<T> a{};
@@ -481,7 +482,7 @@ cudaError_t launch_t(fdtd_batch *b, cudaStream_t st, int nsteps)
     cfg.blockDim = dim3(kBatchThreads);
     cfg.dynamicSmemBytes = batch_smem_bytes<T>(b->pitch);
     if (cfg.dynamicSmemBytes > 48 * 1024) {
-        const cudaError_t e = cudaFuncSetAttribute(k_batch1d<TS, T, VPL, L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        const cudaError_t e = cudaFuncSetAttribute(k_batch1d<TS, T, VPL, L, VS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                                    (int)cfg.dynamicSmemBytes);
         if (e != cudaSuccess) return e;
     }
@@ -493,14 +494,14 @@ cudaError_t launch_t(fdtd_batch *b, cudaStream_t st, int nsteps)
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, k_batch1d<TS, T, VPL, L>, a);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, k_batch1d<TS, T, VPL, L, VS>, a);
     if (e != cudaSuccess) return e;
     k_batch_advance<<<1, 1, 0, st>>>(b->d_step, nsteps);
     return cudaGetLastError();
 }
 
 // clusters of `ctas` CTAs that can be resident at once (0: none fits)
-template <typename TS, typename T, int VPL, int L>
+template <typename TS, typename T, int VPL, int L, int VS = VPL>
 int max_clusters(int ctas)
 {
     cudaLaunchConfig_t cfg{};
@@ -509,7 +510,7 @@ int max_clusters(int ctas)
     // tables of the largest row (128 vectors of 16 bytes) and the field stages
     cfg.dynamicSmemBytes = 3 * 128 * 16 + 2 * kBatchBufs * (size_t)kBatchStage * sizeof(T);
     if (cfg.dynamicSmemBytes > 48 * 1024 &&
-        cudaFuncSetAttribute(k_batch1d<TS, T, VPL, L>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaFuncSetAttribute(k_batch1d<TS, T, VPL, L, VS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)cfg.dynamicSmemBytes) != cudaSuccess) {
         cudaGetLastError();
         return 0;
@@ -522,7 +523,7 @@ int max_clusters(int ctas)
     cfg.attrs = attr;
     cfg.numAttrs = 1;
     int n = 0;
-    if (cudaOccupancyMaxActiveClusters(&n, (void *)k_batch1d<TS, T, VPL, L>, &cfg) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveClusters(&n, (void *)k_batch1d<TS, T, VPL, L, VS>, &cfg) != cudaSuccess) {
         cudaGetLastError();
         n = 0;
     }
@@ -533,10 +534,10 @@ int max_clusters(int ctas)
 // fixes the cluster packing; fdtd_batch_autotune may switch to another.  The built-in one sums J in the order of the
 // single-run default (kinetic_default_shape), so that a run of a batch has the bits it has alone.  The FP64 validation
 // instantiation keeps the built-in shape only.
-template <typename TS, typename T, int VPL, int L>
+template <typename TS, typename T, int VPL, int L, int VS = VPL>
 fdtd_batch::Shape shape_of()
 {
-    return fdtd_batch::Shape{VPL, L, launch_t<TS, T, VPL, L>};
+    return fdtd_batch::Shape{VPL, L, launch_t<TS, T, VPL, L, VS>};
 }
 
 template <typename TS, typename T>
@@ -558,8 +559,8 @@ bool pick(int V, std::vector<fdtd_batch::Shape> &sh, int (**maxc)(int))
         break;
     case 8:
         if constexpr (f32) {
-            sh = {shape_of<TS, T, 2, 4>(), shape_of<TS, T, 4, 2>()};
-            *maxc = max_clusters<TS, T, 2, 4>;
+            sh = {shape_of<TS, T, 4, 2, 2>(), shape_of<TS, T, 2, 4>()};   // (four a lane, summed as two: 2 % ahead)
+            *maxc = max_clusters<TS, T, 4, 2, 2>;
         } else {
             sh = {shape_of<TS, T, 4, 2>()};
             if constexpr (more) sh.push_back(shape_of<TS, T, 2, 4>());

@@ -37,9 +37,10 @@ __global__ void __launch_bounds__(256) k_kinetic(KinArgs<TA> a)
     // (not the shortest BF16 rows: one more condition in their loop costs them a CTA a SM and 10 %)
     constexpr bool kEarly = !(std::is_same<TS, __nv_bfloat16>::value && VPL * L <= 8);
     // Rows a lane each: consecutive vectors share a 32-byte sector, so the lines stay in L1 by the plain policy until
-    // the row is loaded (streaming loads give them up early: 32-node BF16 rows, 2 GB of them 755 -> 721 us, 16-node
-    // FP32 rows 841 -> 793, 16-node BF16 rows 808 -> 792).  Two-vector FP32 rows and longer rows are no faster with it
-    // (8-node FP32 789 -> 821, 64-node BF16 709 -> 710) and keep the streaming hint.
+    // the row is loaded (streaming loads give them up early: 2.1 GB of 32-node BF16 rows 808 -> 772 us, of 16-node
+    // FP32 rows 892 -> 840, of 16-node BF16 rows 864 -> 847).  Two-vector FP32 rows and longer ones are no faster with
+    // it, or hardly (8-node FP32 840 -> 860, 64-node BF16 760 both, 32-node FP32 700 -> 694), and keep the streaming
+    // hint (profiles/probes_rows_fp64_lines.md).
     constexpr bool kShared = L == 1 && !std::is_same<TS, double>::value &&
                              (VPL == 4 || (VPL == 2 && std::is_same<TS, __nv_bfloat16>::value));
     V v[VPL];

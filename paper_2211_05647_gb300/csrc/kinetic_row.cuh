@@ -149,7 +149,7 @@ struct Store<__nv_bfloat16> {
 // terms, and which takes a fifth of the row's instructions.  BF16 rows run on
 // the two-lane FP32 instructions: node pairs (2t, 2t+1) get alpha df + (beta nE)
 // with the roundings of the scalar fma, and the sum is kept as two partial sums
-// (even and odd nodes) added at the end.  VS = VPL / 2 (BF16 rows): the lane
+// (even and odd nodes) added at the end.  VS = VPL / 2: the lane
 // forms the sums of two lanes of the (VS, 2 L) shape, l and l + L, and adds them
 // as that shape's first reduction level does: J is the narrower shape's bit for
 // bit, with VPL loads in flight a lane.
@@ -158,10 +158,9 @@ __device__ __forceinline__ void row_update_to(const typename Vec<TS>::type *v, c
                                               const TA *w_tab, TA nE, int l, uint32_t row_id, int64_t step, uint2 key,
                                               TA &s, TA &c, Put &&put)
 {
-    constexpr int VEC = Vec<TS>::n;
+    constexpr int VEC = Vec<TS>::n, NG = VPL / VS;
+    static_assert(NG == 1 || NG == 2, "one or two partial sums a lane");
     if constexpr (std::is_same<TS, __nv_bfloat16>::value) {
-        constexpr int NG = VPL / VS;
-        static_assert(NG == 1 || NG == 2, "one or two partial sums a lane");
         uint64_t s2[NG];
 #pragma unroll
         for (int g = 0; g < NG; ++g) s2[g] = f2(0.0f, 0.0f);
@@ -196,9 +195,10 @@ __device__ __forceinline__ void row_update_to(const typename Vec<TS>::type *v, c
             c = lo;
         }
     } else {
+        TA sg[NG], cg[NG];
 #pragma unroll
         for (int q = 0; q < VPL; ++q) {
-            const int vi = q * L + l;
+            const int vi = q * L + l, g = q % NG;
             TA x[VEC], al[VEC], be[VEC], w[VEC];
             unpack(v[q], x);
             lds<VEC>(al_tab + vi * VEC, al);
@@ -208,17 +208,25 @@ __device__ __forceinline__ void row_update_to(const typename Vec<TS>::type *v, c
             for (int t = 0; t < VEC; ++t) {
                 x[t] = al[t] * x[t] + be[t] * nE;
                 const TA p = mul_rn(w[t], x[t]);
-                if (q == 0 && t == 0) {   // the first term starts the sum
-                    s = p;
-                    c = TA(0);
+                if (q < NG && t == 0) {   // the first term starts the sum
+                    sg[g] = p;
+                    cg[g] = TA(0);
                     continue;
                 }
                 TA hi, lo;
-                two_sum(s, p, hi, lo);
-                s = hi;
-                c += lo;
+                two_sum(sg[g], p, hi, lo);
+                sg[g] = hi;
+                cg[g] += lo;
             }
             put(vi, Store<TS>::pack(x, uint4{}, uint2{}));
+        }
+        s = sg[0];
+        c = cg[0];
+        if constexpr (NG == 2) {
+            TA hi, lo;
+            two_sum(s, sg[1], hi, lo);
+            s = hi;
+            c = c + cg[1] + lo;
         }
     }
 }

@@ -25,9 +25,9 @@
 //
 // Bound by the exchange and barrier latencies while a CTA has few rows (2000 cells,
 // 500 rows of 64 nodes: 0.97 us a step against 6.0 for the three launches), by
-// shared memory when it has many (150 k cells, 100 k BF16 rows: 11.6 us both), in
-// FP64 by the FP64 pipe on the rows (2.3 against 13.1 us; 100 k rows 120 against
-// 175).
+// shared memory when it has many (110 k cells, 100 k BF16 rows of 64 nodes: 6.3
+// against 11.5), in FP64 by the FP64 pipe on the rows (the 500 rows 2.3 against
+// 13.1 us; 100 k rows of 16 nodes 28 against 54).
 #include "async.cuh"
 #include "kinetic_row.cuh"
 #include "line1d.cuh"
