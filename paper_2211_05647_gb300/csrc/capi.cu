@@ -814,8 +814,9 @@ cudaError_t enqueue(fdtd_plasma *h, cudaStream_t st, int nsteps)
 // per SM; rows of up to 128 sixteen-byte vectors) steps through the cooperative kernel of line1d.cu; what reads
 // or adds to a step from outside (ports, the recorder, the closure) and the nonlinear and evolving-F0 rows take
 // the step graphs.  Measured against the graphs over the sizes that fit: 500 rows of 64 nodes on 2000 cells, FP32
-// 0.97 against 6.0 us a step, FP64 2.3 against 13.1; 30 k rows, FP32 4.9 against 8.0; 100 k BF16 rows 11.6 both
-// (FP32: no longer fits); a million cells without plasma 2.6 against 8.7.  So what fits takes the kernel.
+// 1.0 against 6.0 us a step, FP64 2.3 against 13.1; 30 k rows on 60 k cells, FP32 4.9 against 8.1; 100 k BF16 rows on
+// 110 k cells 6.3 against 11.5 (FP32: no longer fits), FP64 rows of 16 nodes there 28 against 54; a million cells
+// without plasma 2.6 against 8.7.  So what fits takes the kernel.
 // A row shape asked for by option sums J in its own order: only where that is the order of the kernel's rows (the
 // default shape's; in FP64 rows they have a shape of their own) does the kernel take the grid.
 bool line_applies(const fdtd_plasma *h)
@@ -860,12 +861,6 @@ int stream_sms(const fdtd_plasma *h)
     return std::min(h->num_sms, (int)r.sm.smCount);
 }
 
-LinePlan line_plan(const fdtd_plasma *h)
-{
-    // a row weighs its nodes: an FP64 row is bound by the FP64 pipe, and the cells of a range cost next to nothing
-    return line1d_plan(h->nz, h->h_cells, stream_sms(h), h->has_plasma ? (double)h->pitch : 0.0);
-}
-
 // whether the 1-D stepping kernel steps the grid, decided from sizes alone on first use
 bool line_steps(fdtd_plasma *h)
 {
@@ -874,13 +869,20 @@ bool line_steps(fdtd_plasma *h)
         h->line_state = -1;
         const int f_dtype = line_dtype(h), pitch = h->has_plasma ? h->pitch : 0;
         if (pitch / (f_dtype == FDTD_DF_BF16 ? 8 : (f_dtype == FDTD_DF_F64 ? 2 : 4)) > 128) return false;
-        const LinePlan p = line_plan(h);
+        // a row weighs its nodes: an FP64 row is bound by the FP64 pipe, and the cells of a range cost next to nothing
+        LinePlan p = line1d_plan(h->nz, h->h_cells, stream_sms(h), (double)pitch);
         int most = 0;
         if (cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->dev) != cudaSuccess) {
             cudaGetLastError();
             return false;
         }
-        if (line1d_smem_bytes(f_dtype, pitch, p.rows_max, p.nodes_max) + 1024 <= (size_t)most) h->line_state = 1;
+        if (line1d_smem_bytes(f_dtype, pitch, p.rows_max, p.nodes_max) + 1024 > (size_t)most) return false;
+        h->line_ctas = (int)p.cut.size() - 1;
+        h->line_rows = p.rows_max;
+        h->line_nodes = p.nodes_max;
+        h->line_plan = std::move(p.cut);
+        h->line_plan.insert(h->line_plan.end(), p.slot_cut.begin(), p.slot_cut.end());
+        h->line_state = 1;
     }
     return h->line_state > 0;
 }
@@ -888,24 +890,18 @@ bool line_steps(fdtd_plasma *h)
 // the plan and the mailboxes on the device, before the first launch
 int line_prepare(fdtd_plasma *h)
 {
-    const LinePlan p = line_plan(h);
-    const size_t n = p.cut.size();
-    h->line_cut = (int32_t *)dalloc(h, 2 * n * sizeof(int32_t));
-    h->line_mail = (uint64_t *)dalloc(h, (n - 1) * 8 * sizeof(uint64_t));
+    const size_t cuts = h->line_plan.size() * sizeof(int32_t), mail = (size_t)h->line_ctas * 8 * sizeof(uint64_t);
+    h->line_cut = (int32_t *)dalloc(h, cuts);
+    h->line_mail = (uint64_t *)dalloc(h, mail);
     if (!h->line_cut || !h->line_mail) {   // no room: the graphs need none of it
         free_line(h);
         h->err.clear();
         h->line_state = -1;
         return FDTD_OK;
     }
-    std::vector<int32_t> both(p.cut);
-    both.insert(both.end(), p.slot_cut.begin(), p.slot_cut.end());
-    CK(h, cudaMemsetAsync(h->line_mail, 0, (n - 1) * 8 * sizeof(uint64_t), h->stream));
-    CK(h, cudaMemcpyAsync(h->line_cut, both.data(), both.size() * sizeof(int32_t), cudaMemcpyHostToDevice, h->stream));
+    CK(h, cudaMemsetAsync(h->line_mail, 0, mail, h->stream));
+    CK(h, cudaMemcpyAsync(h->line_cut, h->line_plan.data(), cuts, cudaMemcpyHostToDevice, h->stream));
     CK(h, cudaStreamSynchronize(h->stream));
-    h->line_ctas = (int)n - 1;
-    h->line_rows = p.rows_max;
-    h->line_nodes = p.nodes_max;
     h->line_seq = 1;
     return FDTD_OK;
 }

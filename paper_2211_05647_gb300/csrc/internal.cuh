@@ -505,7 +505,8 @@ struct fdtd_plasma {
     // (line_state 0: not looked at yet, 1: the state fits, -1: this configuration takes the step graphs)
     int line_state, line_ctas, line_rows, line_nodes;
     uint32_t line_seq;         // tag of the next launch's first message
-    int32_t *line_cut;         // cut[line_ctas + 1], then slot_cut[line_ctas + 1]
+    std::vector<int32_t> line_plan;   // cut[line_ctas + 1], then slot_cut[line_ctas + 1]
+    int32_t *line_cut;         // the same on the device, from the first launch on
     uint64_t *line_mail;
     // running-DFT ports (device arrays; nports = 0: none)
     int nports, nfreq;
