@@ -346,15 +346,22 @@ int stencil_cpt(const fdtd_plasma *h)
 // the fields no longer live in L2,
 //  2-D whole grids of 6 M cells and more: the fused E + H column march, 4 rows a segment, 8 from 32 M cells
 //      (us a step against the separate passes: 3000^2 51 / 59, 4096^2 80 / 107, 8192^2 263 / 384; 2048^2, in L2,
-//      27 / 24).  Its second field set must stay below a sixteenth of the device's memory.
+//      27 / 24).  Its second field set must stay below a sixteenth of the device's memory, and nine tenths of the
+//      cells must lie inside the layers: a strip that meets a layer runs its slower rows from end to end (layers of 8,
+//      64 x 190 000 cells 209 / 201, 200 000 x 48 88 / 71, 200 x 60 000 137 / 173; of 16, 300 x 40 000 117 / 100;
+//      without layers 64 x 190 000 84 / 96, 24 x 400 000 154 / 179).
 //  3-D grids of 12 M cells and more: the TMA columns, 12 planes a block (256^3 240 / 265, 512^3 1518 / 2019;
-//      192^3 129 / 118).
+//      192^3 129 / 118), where its 8-row blocks are filled to three fifths (640 x 3 x 6666 254 / 175, 640 x 4 x 5000
+//      200 / 166, 640 x 5 x 4000 170 / 191) and more than 4/7 of a plane lies inside the x and y layers (layers of 8,
+//      64 x 64 x 3000 254 / 250, 36 x 36 x 10 000 455 / 444, 512 x 26 x 1000 269 / 264; 64 x 320 x 640 250 / 251).
+//      Narrow rows lose nothing: the cell kernels' blocks are as wide (nx = 4: 903 / 1006).
 // Results are the same bit for bit.
 void default_stencils(fdtd_plasma *h)
 {
     if (h->st_bx > 0 || h->g.precision != FDTD_F32 || h->nx % 4) return;
-    const int64_t cells = h->nx * h->ny * h->nz;
-    if (h->g.ndim == 2 && !h->sd_on && cells >= 6000000) {
+    const int64_t cells = h->nx * h->ny * h->nz, L = h->g.cpml_cells;
+    const double inside = (double)(h->nx - 2 * L) / (double)h->nx * (double)(h->ny - 2 * L) / (double)h->ny;   // of a plane
+    if (h->g.ndim == 2 && !h->sd_on && cells >= 6000000 && inside >= 0.9) {
         size_t avail = 0, total = 0;
         if (cudaMemGetInfo(&avail, &total) != cudaSuccess) {
             cudaGetLastError();
@@ -363,7 +370,7 @@ void default_stencils(fdtd_plasma *h)
         if ((size_t)cells * 3 * 4 > total / 16) return;
         h->auto_fuse_rows = cells >= 32000000 ? 8 : 4;
         h->fuse_by_rule = 1;
-    } else if (h->g.ndim == 3 && cells >= 12000000) {
+    } else if (h->g.ndim == 3 && cells >= 12000000 && 5 * h->ny >= 3 * ((h->ny + 7) / 8 * 8) && inside > 4.0 / 7.0) {
         h->st_tz = 12;   // (the grid-of-cells block keeps its default, for when the option turns the columns off)
     }
 }

@@ -27,8 +27,8 @@ def _equal(a, b, nd):
     assert all(np.array_equal(a.read(q, device=False), b.read(q, device=False)) for q in FIELDS[nd])
 
 
-@pytest.mark.parametrize("dims,cpml,rows", [((24, 262144), 4, None), ((24, 262140), 4, None), ((8, 262141), 2, 4),
-                                            ((8, 65537), 2, 1)])
+@pytest.mark.parametrize("dims,cpml,rows", [((24, 262144), 0, None), ((24, 262140), 0, None),
+                                            ((24, 262144), 4, 4), ((8, 262141), 2, 4), ((8, 65537), 2, 1)])
 def test_march_on_tall_grids(dims, cpml, rows):
     """6.3 M cells take the fused march by the size rule; shorter ones by option with the given rows a segment."""
     a, b = _start(dims, cpml), _start(dims, cpml)
@@ -44,8 +44,24 @@ def test_march_on_tall_grids(dims, cpml, rows):
 def test_cell_kernels_on_deep_grids(dims):
     """12.6 M cells take the TMA columns by the size rule; turned off, the grid-of-cells kernels cover two planes a
     block, as they do on grids the rule leaves alone (one plane a block would need more than 65535 along z)."""
-    a, b = _start(dims, 2), _start(dims, 2)
+    a, b = _start(dims, 0), _start(dims, 0)
     b.set_option("stencil_tz", 0)
     assert a.launch_shapes()["stencil_tz"] > 0 and b.launch_shapes()["stencil_tz"] == 0
     assert b.launch_shapes()["block_z"] == 2
     _equal(a, b, 3)
+
+
+@pytest.mark.parametrize("dims,cpml,fast", [((64, 125000), 8, False), ((64, 125000), 0, True), ((200, 60000), 8, True),
+                                            ((196, 60000), 16, False), ((200000, 48), 8, False), ((640, 3, 6668), 0, False),
+                                            ((640, 4, 5000), 0, False), ((640, 5, 4000), 0, True),
+                                            ((640, 9, 2224), 0, False), ((512, 26, 1000), 8, False),
+                                            ((512, 1000, 26), 8, True), ((64, 64, 3000), 8, False),
+                                            ((64, 320, 640), 8, True)])
+def test_rules_leave_layers_and_thin_grids_alone(dims, cpml, fast):
+    a, b = _start(dims, cpml), _start(dims, cpml)
+    b.set_option("stencil_tz", 0)
+    assert (a.launch_shapes()["fused_rows" if len(dims) == 2 else "stencil_tz"] > 0) == fast
+    for s in (a, b):
+        s.step(4)
+    for q in FIELDS[len(dims)]:
+        assert bool((a.read(q) == b.read(q)).all()), q
