@@ -269,9 +269,10 @@ int fdtd_selftest_line_wait(uint32_t limit_us, int32_t *gave_up);
 
 /* Runtime options.  Without any, and without autotuned or cached shapes, the
  * sizes choose: 2-D FP32 whole grids of 6 M cells and more (nx a multiple of
- * 4) of which nine tenths lie inside the layers run the fused column march below
- * when its second field set (allocated by the first step) fits in a
- * sixteenth of the device's memory, 3-D FP32 grids of 12 M cells and more (ny
+ * 4) of which nine tenths lie inside the layers have the fused column march below
+ * (fdtd_tune_result.fused_rows), which the step sequence runs from 9 M cells, or
+ * from 7.6 M with at most 64 MB of delta f, when its second field set (allocated
+ * by the first step) fits in a sixteenth of the device's memory; 3-D FP32 grids of 12 M cells and more (ny
  * filling blocks of 8 to three fifths, more than 4/7 of a plane inside the x and
  * y layers) the TMA columns of 12 planes, others the grid-of-cells kernels; setting
  * FDTD_OPT_FUSED_STENCILS to 0 or FDTD_OPT_STENCIL_TZ ends the 2-D rule.

@@ -344,8 +344,8 @@ int stencil_cpt(const fdtd_plasma *h)
 
 // Stencils of a handle that the tuning cache knows nothing about (FP32, nx a multiple of 4): from the sizes where
 // the fields no longer live in L2,
-//  2-D whole grids of 6 M cells and more: the fused E + H column march, 4 rows a segment, 8 from 32 M cells
-//      (us a step against the separate passes: 3000^2 51 / 59, 4096^2 80 / 107, 8192^2 263 / 384; 2048^2, in L2,
+//  2-D whole grids of 6 M cells and more, and there where wants_fused says so: the fused E + H column march, 4 rows
+//      a segment, 8 from 32 M cells (us a step against the separate passes: 3000^2 51 / 59, 4096^2 80 / 107, 8192^2 263 / 384; 2048^2, in L2,
 //      27 / 24).  Its second field set must stay below a sixteenth of the device's memory, and nine tenths of the
 //      cells must lie inside the layers: a strip that meets a layer runs its slower rows from end to end (layers of 8,
 //      64 x 190 000 cells 209 / 201, 200 000 x 48 88 / 71, 200 x 60 000 137 / 173; of 16, 300 x 40 000 117 / 100;
@@ -719,10 +719,26 @@ void free_second_set(fdtd_plasma *h)
     for (int q = 0; q < 12; ++q) { dfree(h, h->psi2[q]); h->psi2[q] = nullptr; }
 }
 
+// Whether the step sequence runs the fused pass: by option, by the tuner's choice, or by the size rule
+// (default_stencils) where the fields have left L2.  Below 9 M cells one field set still fits it and the march's two
+// do not, so there the march needs 7.6 M cells and rows whose traffic does not flush the fields anyway, up to 64 MB of
+// delta f (2496^2 with layers of 8: 36 us a step against 31 for the separate passes, 182 / 173 with 400 MB of delta f;
+// 2800^2: 43 / 45, with 40 MB 61 / 64, with 400 MB 193 / 190; 3000^2: 48 / 57, 66 / 75, 202 / 208).
+bool wants_fused(const fdtd_plasma *h)
+{
+    if (h->g.ndim < 2 || h->g.precision != FDTD_F32) return false;
+    if (h->fuse) return true;
+    if (h->g.ndim != 2 || h->auto_fuse_rows <= 0) return false;
+    if (!h->fuse_by_rule) return true;
+    const int64_t cells = h->nx * h->ny;
+    return cells >= 9000000 ||
+           (cells >= 7600000 && h->nkin * (int64_t)h->pitch * (int64_t)h->df_esz <= (int64_t)64 << 20);
+}
+
 // allocate the second field / psi set when the fused sequence applies; on failure the steps run unfused
 void ensure_second_set(fdtd_plasma *h)
 {
-    if ((!h->fuse && h->auto_fuse_rows <= 0) || h->g.ndim < 2 || h->g.precision != FDTD_F32 || h->f2[FDTD_EZ]) return;
+    if (!wants_fused(h) || h->f2[FDTD_EZ]) return;
     bool ok = true;
     for (int q = 0; q < 6 && ok; ++q)
         if (h->flen[q]) ok = (h->f2[q] = dalloc(h, h->flen[q] * h->esz)) != nullptr;
@@ -734,13 +750,8 @@ void ensure_second_set(fdtd_plasma *h)
     }
 }
 
-// whether the step sequence fuses E^{n+1} with H^{n+3/2} (2-D / 3-D FP32 by option, 2-D FP32 by the
-// autotuner's choice; second field set allocated)
-bool fused_stencils(const fdtd_plasma *h)
-{
-    const bool on = h->fuse || (h->auto_fuse_rows > 0 && h->g.ndim == 2);
-    return on && h->g.ndim >= 2 && h->g.precision == FDTD_F32 && h->f2[FDTD_EZ] != nullptr;
-}
+// whether the step sequence fuses E^{n+1} with H^{n+3/2} (second field set allocated)
+bool fused_stencils(const fdtd_plasma *h) { return wants_fused(h) && h->f2[FDTD_EZ] != nullptr; }
 
 // an explicit choice of the separate passes (a stencil option) ends the size rule's fused pass
 void end_fuse_rule(fdtd_plasma *h)
@@ -2047,12 +2058,12 @@ int fdtd_plasma_autotune(fdtd_plasma_t h, fdtd_tune_result *out)
     if (!blob) return fail(h, FDTD_ERR_NOMEM, "autotune: no room for the state copy (%zu bytes)", nb);
     int rc = fdtd_plasma_save_state(h, blob, nb, 1);
     const int64_t steps = h->steps_done;
+    h->fuse_by_rule = 0;   // the tuner's choice from here on
     if (rc == FDTD_OK) rc = h->g.precision == FDTD_F64 ? autotune_t<double>(h, out) : autotune_t<float>(h, out);
     const int rc2 = fdtd_plasma_load_state(h, blob, nb, 1);
     h->steps_done = steps;
     dfree(h, blob);
     drop_graphs(h);
-    h->fuse_by_rule = 0;   // the tuner's choice now
     return rc != FDTD_OK ? rc : rc2;
 }
 

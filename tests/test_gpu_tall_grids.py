@@ -65,3 +65,27 @@ def test_rules_leave_layers_and_thin_grids_alone(dims, cpml, fast):
         s.step(4)
     for q in FIELDS[len(dims)]:
         assert bool((a.read(q) == b.read(q)).all()), q
+
+
+def _allocated(s):
+    return sum(t.numel() for t in s._alloc.live.values())
+
+
+@pytest.mark.parametrize("n,mb,runs", [(2500, 0, False), (2720, 0, False), (2760, 0, True), (2760, 60, True),
+                                       (2760, 70, False), (2996, 70, False), (3004, 70, True)])
+def test_march_runs_where_the_fields_have_left_l2(n, mb, runs):
+    """Between 6 and 9 M cells the march that the size rule names runs from 7.6 M cells and beside little delta f
+    only: the first steps allocate its second field set, or not."""
+    rows = mb << 10   # of 256 FP32 nodes
+    a, b = _start((n, n), 8), _start((n, n), 8)
+    if rows:
+        d = np.zeros(n * n)
+        at = np.arange(n * 100, n * n)
+        d[at[at % n > 0][:rows]] = 1e16
+        for s in (a, b):
+            s.set_plasma(d, vgrid="cart2d", nv=16, nv_perp=16)
+    b.set_option("stencil_tz", 0)
+    assert a.launch_shapes()["fused_rows"] > 0
+    before = _allocated(a)
+    _equal(a, b, 2)
+    assert (_allocated(a) - before >= 12 * n * n) == runs
