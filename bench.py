@@ -250,15 +250,19 @@ def batch_traffic(workload: str, steps_per_launch: int):
     return None
 
 
-def kinetic_kernel(shapes: dict, evolve: bool, fbytes: int = 4, nn: int = 1024, ns: int = 1 << 20):
+def field_bytes(spec: dict, cells: int) -> int:
+    return (8 if spec["grid"].get("precision", "f32") == "f64" else 4) * {1: 2, 2: 3, 3: 6}[spec["grid"]["ndim"]] * cells
+
+
+def kinetic_kernel(shapes: dict, evolve: bool, fbytes: int, nn: int, ns: int, fields: int):
     """The kinetic kernel a handle launches and its launch shape (vpl, l, ring stages); fbytes, nn, ns: the rows an
-    untuned handle's built-in choice follows (the workloads' row lengths)."""
+    untuned handle's built-in choice follows (the workloads' row lengths), with the bytes of the fields."""
     if evolve:
         return "k_kinetic_f0", None
     if shapes["kin_vpl"]:
         shape = (shapes["kin_vpl"], shapes["kin_l"], shapes.get("kin_stages", 0))
     elif fbytes == 4 and nn == 1024:
-        shape = (16, 16, 3 if ns * nn * 4 >= 512 << 20 else 0)
+        shape = (16, 16, 3 if ns * nn * 4 >= 512 << 20 and fields >= 108 << 20 else 0)
     else:
         vecs = max(1, nn * fbytes // 16)
         shape = (min(4, vecs), max(1, vecs // 4), 0)
@@ -350,10 +354,8 @@ def solver_config(workload: str, steps: int, warmup: int, autotune: bool, local:
     evolve = bool(spec["plasma"].get("evolve_f0"))
     alg = 2 * fbytes * ns * nn * (2 if evolve else 1)
     peak, src = _peak()
-    kname, kshape = kinetic_kernel(shapes, evolve, fbytes, nn, ns)
-    fb = 8 if spec["grid"].get("precision", "f32") == "f64" else 4
-    ncomp = {1: 2, 2: 3, 3: 6}[spec["grid"]["ndim"]]
-    step_alg = 2 * fb * ncomp * cells + alg
+    kname, kshape = kinetic_kernel(shapes, evolve, fbytes, nn, ns, field_bytes(spec, cells))
+    step_alg = 2 * field_bytes(spec, cells) + alg
     ms_step = ms / steps
     achieved = alg / (kt["kinetic"] / 1e3) / 1e9
     return {"workload": workload, "steps": steps, "warmup": warmup, "ms_per_step": ms_step,
@@ -755,7 +757,7 @@ def main():
     achieved = alg_bytes / (kt["kinetic"] / 1e3) / 1e9
     peaks = measured_peaks()
     peak = peaks["hbm_gbs"] if peaks else 6800.0
-    kname, kshape = kinetic_kernel(shapes, evolve, fbytes, nn, ns)
+    kname, kshape = kinetic_kernel(shapes, evolve, fbytes, nn, ns, field_bytes(spec, cells))
     roof = {"bound": "hbm", "kernel": kname, "achieved": achieved, "peak": peak, "unit": "GB/s",
             "frac": achieved / peak,
             "traffic": ncu_traffic(kname, args.workload, kshape),

@@ -116,6 +116,7 @@ struct KinArgs {
                                // draws like the whole grid's)
     int store_j;               // k_kinetic: store J^{n+1/2} per slot (the last step of a sequence, or
                                // when something reads it every step); E is updated either way
+    int64_t field_bytes;       // of the grid's E and H (kinetic_default_stages)
     int *err;                  // set to 1 if a bounded wait of the bulk-copy ring kernel gave up
     int after_stencil;         // k_kinetic: what wrote delta f last has ended by the time this launch may start: within
                                // a step sequence another launch, which waits before it lets this one start (pdl_enter),

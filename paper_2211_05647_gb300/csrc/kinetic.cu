@@ -58,21 +58,24 @@ void kinetic_default_shape(int pitch, int f_dtype, int *vpl, int *l)
     *l = V / *vpl;
 }
 
-// How the default shape runs, by the bytes of delta f (same results either way).  Long FP32 rows beyond L2 go
-// through the bulk-copy ring (256 vectors, 3.4 GB: 1.01 against 1.07 ms; 128 and 64, 1.5 GB: 0.468 / 0.465 against
-// 0.480 / 0.477 at two CTAs a SM and 0.500 / 0.491 uncapped); the middle FP32 rows gain from fewer CTAs a SM (16
-// vectors: 0.471 at three against 0.510; 0.3 GB 98 against 104 us).  BF16 rows and the shortest FP32 ones lose with
-// either.
-void kinetic_default_run(int pitch, int f_dtype, int64_t nslots, int l, int *bps, int *stages)
+// How the default shape runs (same results either way): the register kernel, uncapped, or for long FP32 rows beyond L2
+// the bulk-copy ring, by the bytes of delta f and of the fields (us a step, layers of 8, ring / registers).  Rows of 256
+// vectors: where the fields have left L2 too (4096^2 grid, 0.8 GB 331 / 344, 3.4 GB 1090 / 1149; 2048^2, where they have
+// not, 0.6 GB 222 / 215, 3.4 GB 1062 / 1047).  Rows of 64 and 128: where they have not, up to 1 GB (1024^2, 64 vectors,
+// 0.4 GB 141 / 143, 0.8 GB 265 / 276; 2048^2, 0.4 GB 156 / 159, 1.1 GB 392 / 394, 2.3 GB 773 / 759; 4096^2, 0.4 GB
+// 233 / 209, 3.4 GB 1291 / 1160).  A cap on the CTAs a SM, which the middle rows were given before their first loads moved
+// ahead of the grid dependency, only loses since (16 vectors at three CTAs 4096^2, 3.4 GB 1380 / 1205, 1024^2, 40 MB
+// 24.1 / 21.4; 64 at two 1024^2, 40 MB 22.2 / 19.3; the line of 100 k cells with 92 MB of them 29.7 / 24.6).
+int kinetic_default_stages(int pitch, int f_dtype, int64_t nslots, int l, int64_t field_bytes)
 {
-    *bps = *stages = 0;
-    if (f_dtype != FDTD_DF_F32) return;
+    if (f_dtype != FDTD_DF_F32) return 0;
     const int V = pitch / 4;
     const int64_t bytes = nslots * pitch * 4;
-    if (V == 256 && bytes >= (int64_t)512 << 20) *stages = 3;
-    else if ((V == 64 || V == 128) && bytes >= (int64_t)256 << 20) *stages = 4;
-    if (*stages && !kinetic_ring_fits(pitch, f_dtype, l, *stages)) *stages = 0;
-    if (!*stages) *bps = V == 64 || V == 128 ? 2 : (V == 16 || V == 32 ? 3 : 0);
+    const bool fields_in_l2 = field_bytes < (int64_t)108 << 20;   // 9.4 M cells in 2-D, 4.7 M in 3-D
+    int stages = 0;
+    if (V == 256 && bytes >= (int64_t)512 << 20 && !fields_in_l2) stages = 3;
+    else if ((V == 64 || V == 128) && bytes >= (int64_t)256 << 20 && bytes <= (int64_t)1 << 30 && fields_in_l2) stages = 4;
+    return stages && kinetic_ring_fits(pitch, f_dtype, l, stages) ? stages : 0;
 }
 
 cudaError_t dispatch_kinetic_bf16(cudaStream_t st, const KinArgs<float> &a, int num_sms, int vpl, int l, int bps);
@@ -90,7 +93,8 @@ cudaError_t launch_kinetic<float>(cudaStream_t st, const KinArgs<float> &a, int 
         const int V = a.pitch / 8;
         if (f_dtype == FDTD_DF_BF16 && V >= 16 && V <= 128) return dispatch_kinetic_bf16_wide(st, a, num_sms);
         kinetic_default_shape(a.pitch, f_dtype, &vpl, &l);
-        kinetic_default_run(a.pitch, f_dtype, a.nslots, l, &bps, &stages);
+        bps = 0;
+        stages = kinetic_default_stages(a.pitch, f_dtype, a.nslots, l, a.field_bytes);
     }
     if (stages > 0) return launch_kinetic_ring(st, a, f_dtype, num_sms, vpl, l, bps, stages);
     if (f_dtype == FDTD_DF_F32) return dispatch_kinetic<float, float>(st, a, num_sms, vpl, l, bps);

@@ -9,13 +9,14 @@ from tests.adapters import FIELDS
 pytestmark = pytest.mark.gpu
 
 
-#        nodes, delta f (MB), (vectors a lane, lanes)
-@pytest.mark.parametrize("nv,nvp,mb,shape", [(16, 16, 256, (8, 8)), (32, 16, 256, (8, 16)), (32, 32, 512, (16, 16))])
-def test_default_past_the_ring_threshold(nv, nvp, mb, shape, tmp_path, monkeypatch):
+#        nodes, delta f (MB), (vectors a lane, lanes), grid: fields that fit L2, or not
+@pytest.mark.parametrize("nv,nvp,mb,shape,n", [(16, 16, 256, (8, 8), 640), (32, 16, 256, (8, 16), 640),
+                                               (32, 32, 512, (16, 16), 3100)])
+def test_default_past_the_ring_threshold(nv, nvp, mb, shape, n, tmp_path, monkeypatch):
     from paper_2211_05647_gb300 import Solver
     monkeypatch.setenv("FDTD_PLASMA_TUNE_CACHE", str(tmp_path / "none.txt"))
-    rows, n = (mb << 20) // (nv * nvp * 4) + 3, 640
-    spec = spec_2d_cylinder(n=n, R=2, src=(40, 320), nv=nv, nv_perp=nvp, f_dtype="f32", seed=5)
+    rows = (mb << 20) // (nv * nvp * 4) + 3
+    spec = spec_2d_cylinder(n=n, R=2, src=(40, 300), nv=nv, nv_perp=nvp, f_dtype="f32", seed=5)
     d = np.zeros(n * n)
     at = np.arange(n * 60, n * n)
     d[at[at % n > 0][:rows]] = critical_density() * np.linspace(0.05, 0.6, rows)   # (column 0 carries no plasma)
