@@ -332,14 +332,20 @@ dim3 stencil_block(const fdtd_plasma *h)
     return h->g.ndim == 3 ? dim3(32, 4, 2) : dim3(32, 8, 1);
 }
 
-// cells per thread of the curl stencils: tuned, else by size.  2-D: four from 1.5 M cells (2 M cells 16.9 against
-// 18.8 us a step, 4 M 23.6 against 35), one below, where the launch is short and a thread's four cells one after
-// the other make it longer (1 M 11.7 against 10.6, 512^2 8.7 against 4.9).  3-D: one (the four-cell 3-D kernels
-// need 80 registers and lose more to the lower occupancy than they save in instructions).
+// cells per thread of the curl stencils: tuned, else by size.  2-D (FP32, nx a multiple of 4): four on large grids, one
+// below, where the launch is short and a thread's four cells one after the other make it longer.  Where the line lies
+// depends on the layers, which the four-cell kernels' first and last quads of a row meet; layers that fill whole sectors
+// of psi cost them least (us a step, one / four: no layers 640^2 4.5 / 4.7, 800^2 5.9 / 4.8, 1024^2 9.1 / 6.0; layers of
+// 5 1224^2 14.4 / 15.4; of 8 1024^2 10.7 / 11.0, 1160^2 13.2 / 12.4; of 10 1024^2 10.8 / 11.7, 1224^2 14.4 / 13.9; of 16
+// 720^2 6.7 / 6.9, 800^2 7.5 / 6.9, 1024^2 10.8 / 8.5).  3-D: one (the four-cell 3-D kernels need 80 registers and lose
+// more to the lower occupancy than they save in instructions).
 int stencil_cpt(const fdtd_plasma *h)
 {
     if (h->st_cpt > 0) return h->st_cpt;
-    return h->g.ndim == 2 && h->nx * h->ny >= (int64_t)3 << 19 ? 4 : 1;
+    if (h->g.ndim != 2) return 1;
+    const int L = h->g.cpml_cells;
+    const double four_from = L <= 1 || (L >= 16 && L % 8 == 0) ? 0.5e6 : (L == 2 ? 0.75e6 : (L <= 7 ? 1.5e6 : 1.1e6));
+    return (double)h->nx * (double)h->ny >= four_from ? 4 : 1;
 }
 
 // Stencils of a handle that the tuning cache knows nothing about (FP32, nx a multiple of 4): from the sizes where
