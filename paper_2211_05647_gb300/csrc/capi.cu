@@ -399,7 +399,9 @@ KinArgs<T> kin_args(fdtd_plasma *h, int kstep)
     a.kstep = kstep;
     a.slot_base = h->slot_base;
     a.store_j = 1;
-    for (int q = 0; q < 6; ++q) a.field_bytes += h->flen[q] * (int64_t)sizeof(T);
+    a.grid.ndim = h->g.ndim;
+    a.grid.tma = h->g.ndim == 3 && h->st_tz > 0;
+    for (int q = 0; q < 6; ++q) a.grid.field_bytes += h->flen[q] * (int64_t)sizeof(T);
     a.err = h->d_err;
     return a;
 }

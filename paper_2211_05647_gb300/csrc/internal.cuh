@@ -98,6 +98,13 @@ __device__ __forceinline__ double source_value(const Source &s, double t)
     return 0.0;
 }
 
+// what the default way to run the rows follows beside their own size (kinetic_default_run)
+struct KinGrid {
+    int64_t field_bytes;       // of the grid's E and H
+    int ndim;
+    bool tma;                  // the stencils are the TMA columns
+};
+
 template <typename TA>
 struct KinArgs {
     const int32_t *slot_cell;  // polarisation node of each slot
@@ -116,7 +123,7 @@ struct KinArgs {
                                // draws like the whole grid's)
     int store_j;               // k_kinetic: store J^{n+1/2} per slot (the last step of a sequence, or
                                // when something reads it every step); E is updated either way
-    int64_t field_bytes;       // of the grid's E and H (kinetic_default_stages)
+    KinGrid grid;
     int *err;                  // set to 1 if a bounded wait of the bulk-copy ring kernel gave up
     int after_stencil;         // k_kinetic: what wrote delta f last has ended by the time this launch may start: within
                                // a step sequence another launch, which waits before it lets this one start (pdl_enter),

@@ -58,24 +58,33 @@ void kinetic_default_shape(int pitch, int f_dtype, int *vpl, int *l)
     *l = V / *vpl;
 }
 
-// How the default shape runs (same results either way): the register kernel, uncapped, or for long FP32 rows beyond L2
-// the bulk-copy ring, by the bytes of delta f and of the fields (us a step, layers of 8, ring / registers).  Rows of 256
-// vectors: where the fields have left L2 too (4096^2 grid, 0.8 GB 331 / 344, 3.4 GB 1090 / 1149; 2048^2, where they have
-// not, 0.6 GB 222 / 215, 3.4 GB 1062 / 1047).  Rows of 64 and 128: where they have not, up to 1 GB (1024^2, 64 vectors,
-// 0.4 GB 141 / 143, 0.8 GB 265 / 276; 2048^2, 0.4 GB 156 / 159, 1.1 GB 392 / 394, 2.3 GB 773 / 759; 4096^2, 0.4 GB
-// 233 / 209, 3.4 GB 1291 / 1160).  A cap on the CTAs a SM, which the middle rows were given before their first loads moved
-// ahead of the grid dependency, only loses since (16 vectors at three CTAs 4096^2, 3.4 GB 1380 / 1205, 1024^2, 40 MB
-// 24.1 / 21.4; 64 at two 1024^2, 40 MB 22.2 / 19.3; the line of 100 k cells with 92 MB of them 29.7 / 24.6).
-int kinetic_default_stages(int pitch, int f_dtype, int64_t nslots, int l, int64_t field_bytes)
+// How the default shape runs (same results either way): the register kernel, with fewer CTAs a SM where the step before
+// it cannot hide its start, or the bulk-copy ring, for FP32 rows beyond L2 (us a step, layers of 8; 3-D and 1-D without):
+//  1-D, and 3-D behind the TMA columns, which let no successor start early, from 192 MB of delta f: three CTAs a SM for
+//      rows of 16 and 32 vectors, two for 64 and 128 (three / uncapped, 16 vectors, line with 0.6 GB 219 / 233, 256^3
+//      with 2.4 GB 1022 / 1082; two / uncapped, 64 vectors, line with 0.6 GB 200 / 207, 256^3 with 2.4 GB 1010 / 1043).
+//      Elsewhere a cap only loses (16 vectors at three, 4096^2 with 3.4 GB 1380 / 1205, 1024^2 with 40 MB 24.1 / 21.4; 64
+//      at two, 1024^2 with 40 MB 22.2 / 19.3, 128^3 with 1.2 GB 460 / 442).
+//  2-D, fields in L2, 256 MB to 1 GB: the ring for rows of 64 and 128 (ring / registers, 64 vectors, 1024^2 with 0.4 GB
+//      141 / 143, 0.8 GB 265 / 276; 2048^2 with 0.4 GB 156 / 159, 1.1 GB 392 / 394, 2.3 GB 773 / 759; fields beyond L2,
+//      4096^2 with 0.4 GB 233 / 209; 3-D, 128^3 with 0.3 GB 146 / 137).
+//  2-D and 3-D, fields beyond L2, from 512 MB: the ring for rows of 256 (4096^2 with 0.8 GB 331 / 344, 3.4 GB 1090 / 1149;
+//      256^3 with 2.4 GB 998 / 1001; fields in L2, 2048^2 with 0.6 GB 222 / 215, 3.4 GB 1062 / 1047).
+void kinetic_default_run(int pitch, int f_dtype, int64_t nslots, int l, const KinGrid &g, int *bps, int *stages)
 {
-    if (f_dtype != FDTD_DF_F32) return 0;
+    *bps = *stages = 0;
+    if (f_dtype != FDTD_DF_F32) return;
     const int V = pitch / 4;
-    const int64_t bytes = nslots * pitch * 4;
-    const bool fields_in_l2 = field_bytes < (int64_t)108 << 20;   // 9.4 M cells in 2-D, 4.7 M in 3-D
-    int stages = 0;
-    if (V == 256 && bytes >= (int64_t)512 << 20 && !fields_in_l2) stages = 3;
-    else if ((V == 64 || V == 128) && bytes >= (int64_t)256 << 20 && bytes <= (int64_t)1 << 30 && fields_in_l2) stages = 4;
-    return stages && kinetic_ring_fits(pitch, f_dtype, l, stages) ? stages : 0;
+    const int64_t mb = nslots * pitch * 4 >> 20;
+    const bool fields_in_l2 = g.field_bytes < (int64_t)108 << 20;   // 9.4 M cells in 2-D, 4.7 M in 3-D
+    if (V == 256) {
+        if (g.ndim > 1 && mb >= 512 && !fields_in_l2) *stages = 3;
+    } else if (g.ndim == 2) {
+        if ((V == 64 || V == 128) && mb >= 256 && mb <= 1024 && fields_in_l2) *stages = 4;
+    } else if ((g.ndim == 1 || g.tma) && mb >= 192) {
+        *bps = V == 64 || V == 128 ? 2 : (V == 16 || V == 32 ? 3 : 0);
+    }
+    if (*stages && !kinetic_ring_fits(pitch, f_dtype, l, *stages)) *stages = 0;
 }
 
 cudaError_t dispatch_kinetic_bf16(cudaStream_t st, const KinArgs<float> &a, int num_sms, int vpl, int l, int bps);
@@ -93,8 +102,7 @@ cudaError_t launch_kinetic<float>(cudaStream_t st, const KinArgs<float> &a, int 
         const int V = a.pitch / 8;
         if (f_dtype == FDTD_DF_BF16 && V >= 16 && V <= 128) return dispatch_kinetic_bf16_wide(st, a, num_sms);
         kinetic_default_shape(a.pitch, f_dtype, &vpl, &l);
-        bps = 0;
-        stages = kinetic_default_stages(a.pitch, f_dtype, a.nslots, l, a.field_bytes);
+        kinetic_default_run(a.pitch, f_dtype, a.nslots, l, a.grid, &bps, &stages);
     }
     if (stages > 0) return launch_kinetic_ring(st, a, f_dtype, num_sms, vpl, l, bps, stages);
     if (f_dtype == FDTD_DF_F32) return dispatch_kinetic<float, float>(st, a, num_sms, vpl, l, bps);
