@@ -446,7 +446,7 @@ int fdtd_plasma_set_recording(fdtd_plasma_t h, float *samples, int64_t capacity,
  *   loss_grad: loss = mean (y - target)^2 and its gradient (packed like the
  *              parameters, overwritten) -- forward and backward contractions
  *              on BF16 tensor-core tiles with FP32 accumulation, four CTAs per
- *              128-row tile, the tiles' gradients summed in a fixed order
+ *              128-row tile (one where the tiles fill the SMs), the tiles' gradients summed in a fixed order
  *              (deterministic); workspace of fdtd_mlp_workspace_bytes(batch)
  *              bytes (a gradient and the rows of each 128-row tile, about 88 KB, and
  *              the BF16 weights, 80 KB)

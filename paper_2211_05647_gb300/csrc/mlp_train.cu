@@ -1,6 +1,6 @@
 // mlp_train.cu -- loss and gradient of the closure network on the tensor
-// cores: a cluster of four CTAs per 128-row tile of the batch runs the forward
-// pass and the whole backward pass of its tile on mma.sync BF16 tiles with FP32
+// cores: a cluster of four CTAs per 128-row tile of the batch (batches of many
+// tiles: one CTA) runs the forward pass and the whole backward pass of its tile on mma.sync BF16 tiles with FP32
 // accumulation, and writes the tile's gradient; a second kernel sums the tiles'
 // gradients in a fixed order.
 //
@@ -183,6 +183,33 @@ __device__ __forceinline__ void warp_colsum(float *dst, int col, float v0, float
     if (lane < 4) {
         dst[col] = v0;
         dst[col + 1] = v1;
+    }
+}
+
+// a tile's sums over its eight 16-row groups: dW3, db2, db1; db3 and the loss
+__device__ __forceinline__ void tile_colsums(const float (*colsum)[8][kMlpH], const float *loss, const float *dyb,
+                                             float *out, int tid)
+{
+    if (tid < kMlpH) {
+        float a = 0.0f, b = 0.0f, c = 0.0f;
+#pragma unroll
+        for (int w = 0; w < 8; ++w) {
+            a += colsum[0][w][tid];
+            b += colsum[1][w][tid];
+            c += colsum[2][w][tid];
+        }
+        out[kOffW3 + tid] = a;
+        out[kOffB2 + tid] = b;
+        out[kOffB1 + tid] = c;
+    }
+    if (tid == 0) {
+        float l = 0.0f, d = 0.0f;
+        for (int w = 0; w < 8; ++w) {
+            l += loss[w];
+            d += dyb[w];
+        }
+        out[kOffB3] = d;
+        out[kMlpNParams] = l;
     }
 }
 
@@ -428,28 +455,237 @@ __global__ void __cluster_dims__(kTrainCtas, 1, 1) __launch_bounds__(256, 1)
     }
 
     // ---- column sums over the 16-row groups: dW3, db2, db1; db3 and the loss
-    if (rank != 0) return;
-    if (tid < kMlpH) {
-        float a = 0.0f, b = 0.0f, c = 0.0f;
+    if (rank == 0) tile_colsums(s.colsum, s.loss, s.dyb, out, tid);
+}
+
+// The same for batches of more tiles than a wave of clusters takes (launch_train_tile): one tile a CTA, a warp its 16
+// rows through every phase, nothing exchanged between CTAs.  The values are the cluster's, sum for sum.  Bound by the
+// tile's phases as the cluster is (262 144 rows, 2048 tiles: 0.35 ms a minibatch, 80 TFLOP/s).
+struct MlpTrainSmem1 {
+    TrainWeights w;
+    TrainTile t;
+    __nv_bfloat16 h1[kMlpRows][kLd2];     // h1, later dz1 (once dW2 is formed)
+    __nv_bfloat16 dz2[kMlpRows][kLd2];
+    float b1[kMlpH], b2[kMlpH], w3[kMlpH];
+    float colsum[3][8][kMlpH];            // per warp: dW3, db2, db1 partial column sums
+    float loss[8], dyb[8];
+    float b3;
+};
+
+__global__ void __launch_bounds__(256, 1) k_mlp_train_tile1(const float *__restrict__ P, TrainWs ws, int64_t B)
+{
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    MlpTrainSmem1 &s = *reinterpret_cast<MlpTrainSmem1 *>(smem_raw);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int g = lane >> 2, t = lane & 3;
+    const int r0 = warp * 16;
+    const int64_t tile = blockIdx.x;
+    float *out = ws.grad + tile * kTrainStride;
+
+    pdl_enter();
+    const unsigned char *gw = reinterpret_cast<const unsigned char *>(ws.w);
+    const unsigned char *gx = reinterpret_cast<const unsigned char *>(ws.x + tile);
+    for (int i = tid; i < (int)(sizeof(TrainTile) / 16); i += 256)
+        cpa16(reinterpret_cast<unsigned char *>(&s.t) + 16 * i, gx + 16 * i);
+    for (int i = tid; i < (int)(sizeof(TrainWeights) / 16); i += 256)
+        cpa16(reinterpret_cast<unsigned char *>(&s.w) + 16 * i, gw + 16 * i);
+    cpa_commit();
+    const int64_t row = tile * kMlpRows + r0 + g;   // the thread's rows: row and row + 8
+    const float ta = row < B ? ws.t[row] : 0.0f, tb = row + 8 < B ? ws.t[row + 8] : 0.0f;
+    for (int i = tid; i < kMlpH; i += 256) {
+        s.b1[i] = P[kOffB1 + i];
+        s.b2[i] = P[kOffB2 + i];
+        s.w3[i] = P[kOffW3 + i];
+    }
+    if (tid == 0) s.b3 = P[kOffB3];
+    cpa_wait_all();
+    __syncthreads();
+
+    // ---- forward, layer 1: h1 = gelu(z1) -> shared (BF16)
+    uint32_t xa[2][4];   // the warp's rows of x as A fragments (K = 32: two k steps)
 #pragma unroll
-        for (int w = 0; w < 8; ++w) {
-            a += s.colsum[0][w][tid];
-            b += s.colsum[1][w][tid];
-            c += s.colsum[2][w][tid];
-        }
-        out[kOffW3 + tid] = a;
-        out[kOffB2 + tid] = b;
-        out[kOffB1 + tid] = c;
+    for (int ks = 0; ks < kMlpK1 / 16; ++ks) {
+        xa[ks][0] = ld_b32(&s.t.x[r0 + g][ks * 16 + 2 * t]);
+        xa[ks][1] = ld_b32(&s.t.x[r0 + g + 8][ks * 16 + 2 * t]);
+        xa[ks][2] = ld_b32(&s.t.x[r0 + g][ks * 16 + 2 * t + 8]);
+        xa[ks][3] = ld_b32(&s.t.x[r0 + g + 8][ks * 16 + 2 * t + 8]);
     }
-    if (tid == 0) {
-        float l = 0.0f, d = 0.0f;
-        for (int w = 0; w < 8; ++w) {
-            l += s.loss[w];
-            d += s.dyb[w];
-        }
-        out[kOffB3] = d;
-        out[kMlpNParams] = l;
+    auto z1_tile = [&](int nt, float (&z)[4]) {
+        z[0] = z[1] = z[2] = z[3] = 0.0f;
+#pragma unroll
+        for (int ks = 0; ks < kMlpK1 / 16; ++ks)
+            mma_bf16_16816(z, xa[ks], ld_b32(&s.w.w1t[nt * 8 + g][ks * 16 + 2 * t]),
+                           ld_b32(&s.w.w1t[nt * 8 + g][ks * 16 + 2 * t + 8]));
+        const int col = nt * 8 + 2 * t;
+        z[0] += s.b1[col];
+        z[1] += s.b1[col + 1];
+        z[2] += s.b1[col];
+        z[3] += s.b1[col + 1];
+    };
+#pragma unroll
+    for (int nt = 0; nt < 16; ++nt) {
+        float z[4];
+        z1_tile(nt, z);
+        const int col = nt * 8 + 2 * t;
+        *reinterpret_cast<uint32_t *>(&s.h1[r0 + g][col]) = pack_bf16(gelu_f(z[0]), gelu_f(z[1]));
+        *reinterpret_cast<uint32_t *>(&s.h1[r0 + g + 8][col]) = pack_bf16(gelu_f(z[2]), gelu_f(z[3]));
     }
+    __syncwarp();
+
+    // ---- forward, layer 2 (the warp's own rows of h1) and the output y
+    float z2[16][4];
+#pragma unroll
+    for (int nt = 0; nt < 16; ++nt) z2[nt][0] = z2[nt][1] = z2[nt][2] = z2[nt][3] = 0.0f;
+#pragma unroll 2
+    for (int ks = 0; ks < kMlpH / 16; ++ks) {
+        uint32_t a[4];
+        a[0] = ld_b32(&s.h1[r0 + g][ks * 16 + 2 * t]);
+        a[1] = ld_b32(&s.h1[r0 + g + 8][ks * 16 + 2 * t]);
+        a[2] = ld_b32(&s.h1[r0 + g][ks * 16 + 2 * t + 8]);
+        a[3] = ld_b32(&s.h1[r0 + g + 8][ks * 16 + 2 * t + 8]);
+#pragma unroll
+        for (int nt = 0; nt < 16; ++nt)
+            mma_bf16_16816(z2[nt], a, ld_b32(&s.w.w2t[nt * 8 + g][ks * 16 + 2 * t]),
+                           ld_b32(&s.w.w2t[nt * 8 + g][ks * 16 + 2 * t + 8]));
+    }
+    float y0 = 0.0f, y1 = 0.0f;
+#pragma unroll
+    for (int nt = 0; nt < 16; ++nt) {
+        const int col = nt * 8 + 2 * t;
+        z2[nt][0] += s.b2[col];
+        z2[nt][1] += s.b2[col + 1];
+        z2[nt][2] += s.b2[col];
+        z2[nt][3] += s.b2[col + 1];
+        y0 += gelu_f(z2[nt][0]) * s.w3[col] + gelu_f(z2[nt][1]) * s.w3[col + 1];
+        y1 += gelu_f(z2[nt][2]) * s.w3[col] + gelu_f(z2[nt][3]) * s.w3[col + 1];
+    }
+    y0 += __shfl_xor_sync(0xffffffffu, y0, 1);
+    y0 += __shfl_xor_sync(0xffffffffu, y0, 2);
+    y1 += __shfl_xor_sync(0xffffffffu, y1, 1);
+    y1 += __shfl_xor_sync(0xffffffffu, y1, 2);
+    const float e0 = row < B ? y0 + s.b3 - ta : 0.0f;
+    const float e1 = row + 8 < B ? y1 + s.b3 - tb : 0.0f;
+    const float dy0 = 2.0f * e0 / (float)B, dy1 = 2.0f * e1 / (float)B;
+
+    // ---- dW3 = h2^T dy, dz2 = dy w3 GELU'(z2) (-> shared, BF16), db2 = colsum dz2
+#pragma unroll
+    for (int nt = 0; nt < 16; ++nt) {
+        const int col = nt * 8 + 2 * t;
+        warp_colsum(s.colsum[0][warp], col, gelu_f(z2[nt][0]) * dy0 + gelu_f(z2[nt][2]) * dy1,
+                    gelu_f(z2[nt][1]) * dy0 + gelu_f(z2[nt][3]) * dy1, lane);
+        const float d00 = dy0 * s.w3[col] * gelu_grad_f(z2[nt][0]);
+        const float d01 = dy0 * s.w3[col + 1] * gelu_grad_f(z2[nt][1]);
+        const float d10 = dy1 * s.w3[col] * gelu_grad_f(z2[nt][2]);
+        const float d11 = dy1 * s.w3[col + 1] * gelu_grad_f(z2[nt][3]);
+        warp_colsum(s.colsum[1][warp], col, d00 + d10, d01 + d11, lane);
+        *reinterpret_cast<uint32_t *>(&s.dz2[r0 + g][col]) = pack_bf16(d00, d01);
+        *reinterpret_cast<uint32_t *>(&s.dz2[r0 + g + 8][col]) = pack_bf16(d10, d11);
+    }
+    {
+        float l = e0 * e0 + e1 * e1, d = dy0 + dy1;
+        if (t != 0) l = d = 0.0f;   // every lane of a quad holds the same two rows
+#pragma unroll
+        for (int off = 16; off > 0; off >>= 1) {
+            l += __shfl_xor_sync(0xffffffffu, l, off);
+            d += __shfl_xor_sync(0xffffffffu, d, off);
+        }
+        if (lane == 0) {
+            s.loss[warp] = l / (float)B;
+            s.dyb[warp] = d;
+        }
+    }
+    __syncthreads();
+
+    const int q3 = lane >> 3, rr = lane & 7;
+    // ---- dW2[k][n] = sum_b h1[b][k] dz2[b][n]: the warp forms rows k in [16 warp, +16)
+    {
+        float acc[16][4];
+#pragma unroll
+        for (int nt = 0; nt < 16; ++nt) acc[nt][0] = acc[nt][1] = acc[nt][2] = acc[nt][3] = 0.0f;
+#pragma unroll 2
+        for (int ks = 0; ks < kMlpRows / 16; ++ks) {
+            const int b0 = ks * 16;
+            uint32_t a[4];   // A(k, b) = h1[b][k]: blocks (b lo/hi) x (k lo/hi) in the a0..a3 order
+            ldsm_x4_trans(a, &s.h1[b0 + ((q3 >> 1) << 3) + rr][r0 + ((q3 & 1) << 3)]);
+#pragma unroll
+            for (int nt = 0; nt < 16; nt += 2) {
+                uint32_t bq[4];   // B(b, n) = dz2[b][n]: (nt, b lo), (nt, b hi), (nt + 1, b lo), (nt + 1, b hi)
+                ldsm_x4_trans(bq, &s.dz2[b0 + ((q3 & 1) << 3) + rr][(nt + (q3 >> 1)) * 8]);
+                mma_bf16_16816(acc[nt], a, bq[0], bq[1]);
+                mma_bf16_16816(acc[nt + 1], a, bq[2], bq[3]);
+            }
+        }
+#pragma unroll
+        for (int nt = 0; nt < 16; ++nt) {
+            const int col = nt * 8 + 2 * t;
+            float *o = out + kOffW2 + (r0 + g) * kMlpH + col;
+            *reinterpret_cast<float2 *>(o) = make_float2(acc[nt][0], acc[nt][1]);
+            *reinterpret_cast<float2 *>(o + 8 * kMlpH) = make_float2(acc[nt][2], acc[nt][3]);
+        }
+    }
+
+    // ---- dh1 = dz2 W2^T for the warp's own rows, dz1 = dh1 GELU'(z1)
+    float dh[16][4];
+#pragma unroll
+    for (int nt = 0; nt < 16; ++nt) dh[nt][0] = dh[nt][1] = dh[nt][2] = dh[nt][3] = 0.0f;
+#pragma unroll 2
+    for (int ks = 0; ks < kMlpH / 16; ++ks) {
+        uint32_t a[4];
+        a[0] = ld_b32(&s.dz2[r0 + g][ks * 16 + 2 * t]);
+        a[1] = ld_b32(&s.dz2[r0 + g + 8][ks * 16 + 2 * t]);
+        a[2] = ld_b32(&s.dz2[r0 + g][ks * 16 + 2 * t + 8]);
+        a[3] = ld_b32(&s.dz2[r0 + g + 8][ks * 16 + 2 * t + 8]);
+#pragma unroll
+        for (int nt = 0; nt < 16; ++nt)
+            mma_bf16_16816(dh[nt], a, ld_b32(&s.w.w2n[nt * 8 + g][ks * 16 + 2 * t]),
+                           ld_b32(&s.w.w2n[nt * 8 + g][ks * 16 + 2 * t + 8]));
+    }
+    __syncthreads();   // every warp has read h1 (dW2) before dz1 takes its place
+#pragma unroll
+    for (int nt = 0; nt < 16; ++nt) {
+        const int col = nt * 8 + 2 * t;
+        float z[4];
+        z1_tile(nt, z);
+        const float d00 = dh[nt][0] * gelu_grad_f(z[0]), d01 = dh[nt][1] * gelu_grad_f(z[1]);
+        const float d10 = dh[nt][2] * gelu_grad_f(z[2]), d11 = dh[nt][3] * gelu_grad_f(z[3]);
+        warp_colsum(s.colsum[2][warp], col, d00 + d10, d01 + d11, lane);
+        *reinterpret_cast<uint32_t *>(&s.h1[r0 + g][col]) = pack_bf16(d00, d01);
+        *reinterpret_cast<uint32_t *>(&s.h1[r0 + g + 8][col]) = pack_bf16(d10, d11);
+    }
+    __syncthreads();
+
+    // ---- dW1[k][n] = sum_b x[b][k] dz1[b][n] (k < 17): the warp forms the 16-row block k in [16 (warp & 1), +16) for
+    //      the n tiles [4 (warp >> 1), +4)
+    {
+        const int mt = warp & 1, n0 = (warp >> 1) * 4;
+        float acc[4][4];
+#pragma unroll
+        for (int j = 0; j < 4; ++j) acc[j][0] = acc[j][1] = acc[j][2] = acc[j][3] = 0.0f;
+#pragma unroll 2
+        for (int ks = 0; ks < kMlpRows / 16; ++ks) {
+            const int b0 = ks * 16;
+            uint32_t a[4];
+            ldsm_x4_trans(a, &s.t.x[b0 + ((q3 >> 1) << 3) + rr][mt * 16 + ((q3 & 1) << 3)]);
+#pragma unroll
+            for (int j = 0; j < 4; j += 2) {
+                uint32_t bq[4];
+                ldsm_x4_trans(bq, &s.h1[b0 + ((q3 & 1) << 3) + rr][(n0 + j + (q3 >> 1)) * 8]);
+                mma_bf16_16816(acc[j], a, bq[0], bq[1]);
+                mma_bf16_16816(acc[j + 1], a, bq[2], bq[3]);
+            }
+        }
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const int col = (n0 + j) * 8 + 2 * t;
+            const int k_lo = mt * 16 + g, k_hi = k_lo + 8;
+            if (k_lo < kMlpIn)
+                *reinterpret_cast<float2 *>(out + kOffW1 + k_lo * kMlpH + col) = make_float2(acc[j][0], acc[j][1]);
+            if (k_hi < kMlpIn)
+                *reinterpret_cast<float2 *>(out + kOffW1 + k_hi * kMlpH + col) = make_float2(acc[j][2], acc[j][3]);
+        }
+    }
+
+    tile_colsums(s.colsum, s.loss, s.dyb, out, tid);
 }
 
 // grad[i] = sum over tiles (in tile order) of ws[tile][i]; loss = sum of ws[tile][kMlpNParams]
@@ -517,12 +753,21 @@ cudaError_t launch_train_prepare(cudaStream_t st, const float *P, const float *X
                       0, st, P, X, T, B, tiles * kMlpRows, copies, ws, perm ? *perm : Perm{}, perm ? 1 : 0);
 }
 
+// A cluster takes a tile in some 11 us, a CTA in some 20, on a quarter of the SMs: the clusters are ahead while one wave
+// of them does (us a minibatch of an epoch, clusters / CTAs: 32 tiles 18.2 / 25.2, 48 27.4 / 28.1, 64 28.3 / 27.8,
+// 76 36.9 / 30.8, 128 43.4 / 29.9, 512 138 / 87.9, 2048 556 / 352).
 cudaError_t launch_train_tile(cudaStream_t st, const float *P, int64_t B, const TrainWs &ws, int64_t tiles)
 {
-    const size_t smem = sizeof(MlpTrainSmem);
-    cudaError_t e = cudaFuncSetAttribute(k_mlp_train_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
-    return launch_pdl(k_mlp_train_tile, dim3((unsigned)tiles * kTrainCtas), dim3(256), smem, st, P, ws, B);
+    const bool clusters = 8 * tiles <= 3 * sms;
+    const size_t smem = clusters ? sizeof(MlpTrainSmem) : sizeof(MlpTrainSmem1);
+    auto kern = clusters ? k_mlp_train_tile : k_mlp_train_tile1;
+    e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    return launch_pdl(kern, dim3((unsigned)tiles * (clusters ? kTrainCtas : 1)), dim3(256), smem, st, P, ws, B);
 }
 
 }  // namespace fp
