@@ -33,11 +33,11 @@ def test_every_early_launched_kernel_waits():
     launched = set()
     for t in SRC.values():
         for m in re.finditer(r"launch_pdl\(\s*(k_\w+|kern)\b", t):
-            name = m.group(1)
-            if name == "kern":
-                name = re.findall(r"auto kern = (k_\w+)", t[:m.start()])[-1]
-            launched.add(name)
-    assert {"k_kinetic", "k_h2d", "k_e3d", "k_eh2d_v4", "k_copy", "k_kinetic_nl_walk"} <= launched
+            if m.group(1) == "kern":
+                launched |= set(re.findall(r"\bk_\w+", re.findall(r"auto kern = ([^;]*);", t[:m.start()])[-1]))
+            else:
+                launched.add(m.group(1))
+    assert {"k_kinetic", "k_h2d", "k_e3d", "k_eh2d_v4", "k_copy", "k_kinetic_nl_walk", "k_mlp_train_tile1"} <= launched
     for name in launched:
         body = kernels[name]
         assert "pdl_enter()" in body, name
