@@ -896,14 +896,25 @@ bool line_steps(fdtd_plasma *h)
         h->line_state = -1;
         const int f_dtype = line_dtype(h), pitch = h->has_plasma ? h->pitch : 0;
         if (pitch / (f_dtype == FDTD_DF_BF16 ? 8 : (f_dtype == FDTD_DF_F64 ? 2 : 4)) > 128) return false;
-        // a row weighs its nodes: an FP64 row is bound by the FP64 pipe, and the cells of a range cost next to nothing
-        LinePlan p = line1d_plan(h->nz, h->h_cells, stream_sms(h), (double)pitch);
         int most = 0;
         if (cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->dev) != cudaSuccess) {
             cudaGetLastError();
             return false;
         }
-        if (line1d_smem_bytes(f_dtype, pitch, p.rows_max, p.nodes_max) + 1024 > (size_t)most) return false;
+        // What a row weighs in cells of the line: about a third of its nodes where a CTA gets dozens (FP32 and BF16:
+        // a row of 64 nodes takes 9 ns of a step then, a cell 0.4), all of them where it gets few, or in FP64, whose
+        // pipe bounds the rows, or when the ranges of the smaller weight hold too many rows (us a step, third / all:
+        // 25 k rows of 64 nodes on 100 k cells, FP32 2.4 / 4.4, BF16 2.2 / 4.4; 200 of them there, BF16 1.8 / 1.5).
+        const int sms = stream_sms(h);
+        const bool many = f_dtype != FDTD_DF_F64 && (int64_t)h->h_cells.size() >= 32 * (int64_t)sms;
+        LinePlan p;
+        bool fits = false;
+        for (double weight : {many ? 0.36 : 1.0, 1.0}) {
+            p = line1d_plan(h->nz, h->h_cells, sms, std::ceil(weight * (double)pitch));
+            fits = line1d_smem_bytes(f_dtype, pitch, p.rows_max, p.nodes_max) + 1024 <= (size_t)most;
+            if (fits) break;
+        }
+        if (!fits) return false;
         h->line_ctas = (int)p.cut.size() - 1;
         h->line_rows = p.rows_max;
         h->line_nodes = p.nodes_max;
