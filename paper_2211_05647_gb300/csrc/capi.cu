@@ -399,9 +399,6 @@ KinArgs<T> kin_args(fdtd_plasma *h, int kstep)
     a.kstep = kstep;
     a.slot_base = h->slot_base;
     a.store_j = 1;
-    a.grid.ndim = h->g.ndim;
-    a.grid.tma = h->g.ndim == 3 && h->st_tz > 0;
-    for (int q = 0; q < 6; ++q) a.grid.field_bytes += h->flen[q] * (int64_t)sizeof(T);
     a.err = h->d_err;
     return a;
 }
@@ -625,7 +622,9 @@ cudaError_t part_mid(fdtd_plasma *h, cudaStream_t st, int kstep, const FieldSet<
                                      h->sd_on ? h->rows_global : h->nkin);
         } else {
             const KinShape k = kin_shape(h);
-            e = launch_kinetic<T>(st, a, h->pl.f_dtype, h->num_sms, k.vpl, k.l, k.bps, k.stages);
+            KinGrid grid{0, h->g.ndim, h->g.ndim == 3 && h->st_tz > 0};
+            for (int q = 0; q < 6; ++q) grid.field_bytes += h->flen[q] * (int64_t)sizeof(T);
+            e = launch_kinetic<T>(st, a, grid, h->pl.f_dtype, h->num_sms, k.vpl, k.l, k.bps, k.stages);
         }
         if (e != cudaSuccess) return e;
     }

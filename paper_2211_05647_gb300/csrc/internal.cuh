@@ -98,7 +98,8 @@ __device__ __forceinline__ double source_value(const Source &s, double t)
     return 0.0;
 }
 
-// what the default way to run the rows follows beside their own size (kinetic_default_run)
+// what the default way to run the rows follows beside their own size (kinetic_default_run).  Not a part of KinArgs: a
+// longer parameter block moves the row kernels' registers (BF16 rows of 64 nodes 80 to 102, 7 % of their time).
 struct KinGrid {
     int64_t field_bytes;       // of the grid's E and H
     int ndim;
@@ -123,7 +124,6 @@ struct KinArgs {
                                // draws like the whole grid's)
     int store_j;               // k_kinetic: store J^{n+1/2} per slot (the last step of a sequence, or
                                // when something reads it every step); E is updated either way
-    KinGrid grid;
     int *err;                  // set to 1 if a bounded wait of the bulk-copy ring kernel gave up
     int after_stencil;         // k_kinetic: what wrote delta f last has ended by the time this launch may start: within
                                // a step sequence another launch, which waits before it lets this one start (pdl_enter),
@@ -337,8 +337,8 @@ void kinetic_default_shape(int pitch, int f_dtype, int *vpl, int *l);
 // bps > 0 caps the CTAs per SM; stages > 0 (FP32 / BF16 storage) selects the bulk-copy ring kernel
 // with that many shared-memory stages (kinetic_ring.cu)
 template <typename TA>
-cudaError_t launch_kinetic(cudaStream_t st, const KinArgs<TA> &a, int f_dtype, int num_sms, int vpl = 0, int l = 0,
-                           int bps = 0, int stages = 0);
+cudaError_t launch_kinetic(cudaStream_t st, const KinArgs<TA> &a, const KinGrid &grid, int f_dtype, int num_sms,
+                           int vpl = 0, int l = 0, int bps = 0, int stages = 0);
 // whether the ring kernel's tables and stages fit in one CTA's shared memory (FP32 / BF16 rows, stages >= 2)
 bool kinetic_ring_fits(int pitch, int f_dtype, int l, int stages);
 // the bulk-copy ring kernel for an FP32 / BF16 row shape (cudaErrorInvalidValue if the stages do not fit)

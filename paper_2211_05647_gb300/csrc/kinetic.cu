@@ -92,8 +92,8 @@ cudaError_t dispatch_kinetic_bf16_wide(cudaStream_t st, const KinArgs<float> &a,
 cudaError_t dispatch_kinetic_f64(cudaStream_t st, const KinArgs<double> &a, int num_sms, int vpl, int l, int bps);
 
 template <>
-cudaError_t launch_kinetic<float>(cudaStream_t st, const KinArgs<float> &a, int f_dtype, int num_sms, int vpl, int l,
-                                  int bps, int stages)
+cudaError_t launch_kinetic<float>(cudaStream_t st, const KinArgs<float> &a, const KinGrid &grid, int f_dtype,
+                                  int num_sms, int vpl, int l, int bps, int stages)
 {
     if (a.nslots == 0) return cudaSuccess;
     if (vpl <= 0) {
@@ -102,7 +102,7 @@ cudaError_t launch_kinetic<float>(cudaStream_t st, const KinArgs<float> &a, int 
         const int V = a.pitch / 8;
         if (f_dtype == FDTD_DF_BF16 && V >= 16 && V <= 128) return dispatch_kinetic_bf16_wide(st, a, num_sms);
         kinetic_default_shape(a.pitch, f_dtype, &vpl, &l);
-        kinetic_default_run(a.pitch, f_dtype, a.nslots, l, a.grid, &bps, &stages);
+        kinetic_default_run(a.pitch, f_dtype, a.nslots, l, grid, &bps, &stages);
     }
     if (stages > 0) return launch_kinetic_ring(st, a, f_dtype, num_sms, vpl, l, bps, stages);
     if (f_dtype == FDTD_DF_F32) return dispatch_kinetic<float, float>(st, a, num_sms, vpl, l, bps);
@@ -111,8 +111,8 @@ cudaError_t launch_kinetic<float>(cudaStream_t st, const KinArgs<float> &a, int 
 }
 
 template <>
-cudaError_t launch_kinetic<double>(cudaStream_t st, const KinArgs<double> &a, int f_dtype, int num_sms, int vpl, int l,
-                                   int bps, int stages)
+cudaError_t launch_kinetic<double>(cudaStream_t st, const KinArgs<double> &a, const KinGrid &, int f_dtype,
+                                   int num_sms, int vpl, int l, int bps, int stages)
 {
     if (a.nslots == 0) return cudaSuccess;
     if (stages > 0) return cudaErrorInvalidValue;   // the ring kernel streams FP32 / BF16 rows only
