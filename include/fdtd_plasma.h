@@ -272,10 +272,11 @@ int fdtd_selftest_line_wait(uint32_t limit_us, int32_t *gave_up);
  * 4) of which nine tenths lie inside the layers have the fused column march below
  * (fdtd_tune_result.fused_rows), which the step sequence runs from 9 M cells, or
  * from 7.6 M with at most 64 MB of delta f, when its second field set (allocated
- * by the first step) fits in a sixteenth of the device's memory; 3-D FP32 grids of 12 M cells and more (ny
- * filling blocks of 8 to three fifths, more than 4/7 of a plane inside the x and
- * y layers) the TMA columns of 12 planes, others the grid-of-cells kernels; setting
- * FDTD_OPT_FUSED_STENCILS to 0 or FDTD_OPT_STENCIL_TZ ends the 2-D rule.
+ * by the first step) fits in a sixteenth of the device's memory; 3-D FP32 grids
+ * of 12 M cells and more (ny filling blocks of 8 to three fifths, more than 4/7
+ * of a plane inside the x and y layers) run the TMA columns of 12 planes; others
+ * the grid-of-cells kernels.  Setting FDTD_OPT_FUSED_STENCILS to 0 or
+ * FDTD_OPT_STENCIL_TZ ends the 2-D rule.
  * Results are the same bit for bit.
  * FDTD_OPT_FUSED_STENCILS (default 0): 1 makes the step
  * sequence on 2-D and 3-D FP32 grids fuse each E update with the next H update into
@@ -446,8 +447,8 @@ int fdtd_plasma_set_recording(fdtd_plasma_t h, float *samples, int64_t capacity,
  *   loss_grad: loss = mean (y - target)^2 and its gradient (packed like the
  *              parameters, overwritten) -- forward and backward contractions
  *              on BF16 tensor-core tiles with FP32 accumulation, four CTAs per
- *              128-row tile (one where the tiles fill the SMs), the tiles' gradients summed in a fixed order
- *              (deterministic); workspace of fdtd_mlp_workspace_bytes(batch)
+ *              128-row tile (one where the tiles fill the SMs), the tiles' gradients
+ *              summed in a fixed order (deterministic); workspace of fdtd_mlp_workspace_bytes(batch)
  *              bytes (a gradient and the rows of each 128-row tile, about 88 KB, and
  *              the BF16 weights, 80 KB)
  *   adam     : one Adam step (Kingma & Ba, bias-corrected, step count t >= 1)

@@ -350,10 +350,10 @@ int stencil_cpt(const fdtd_plasma *h)
 
 // Stencils of a handle that the tuning cache knows nothing about (FP32, nx a multiple of 4): from the sizes where
 // the fields no longer live in L2,
-//  2-D whole grids of 6 M cells and more, and there where wants_fused says so: the fused E + H column march, 4 rows
-//      a segment, 8 from 32 M cells (us a step against the separate passes: 3000^2 51 / 59, 4096^2 80 / 107, 8192^2 263 / 384; 2048^2, in L2,
-//      27 / 24).  Its second field set must stay below a sixteenth of the device's memory, and nine tenths of the
-//      cells must lie inside the layers: a strip that meets a layer runs its slower rows from end to end (layers of 8,
+//  2-D whole grids of 6 M cells and more, and there where wants_fused says so: the fused E + H column march, 4 rows a
+//      segment, 8 from 32 M cells (us a step against the separate passes: 3000^2 51 / 59, 4096^2 80 / 107, 8192^2
+//      263 / 384; 2048^2, in L2, 27 / 24).  Its second field set must stay below a sixteenth of the device's memory, and
+//      nine tenths of the cells must lie inside the layers: a strip that meets a layer runs its slower rows (layers of 8,
 //      64 x 190 000 cells 209 / 201, 200 000 x 48 88 / 71, 200 x 60 000 137 / 173; of 16, 300 x 40 000 117 / 100;
 //      without layers 64 x 190 000 84 / 96, 24 x 400 000 154 / 179).
 //  3-D grids of 12 M cells and more: the TMA columns, 12 planes a block (256^3 240 / 265, 512^3 1518 / 2019;
@@ -366,7 +366,7 @@ void default_stencils(fdtd_plasma *h)
 {
     if (h->st_bx > 0 || h->g.precision != FDTD_F32 || h->nx % 4) return;
     const int64_t cells = h->nx * h->ny * h->nz, L = h->g.cpml_cells;
-    const double inside = (double)(h->nx - 2 * L) / (double)h->nx * (double)(h->ny - 2 * L) / (double)h->ny;   // of a plane
+    const double inside = (double)(h->nx - 2 * L) / (double)h->nx * (double)(h->ny - 2 * L) / (double)h->ny;
     if (h->g.ndim == 2 && !h->sd_on && cells >= 6000000 && inside >= 0.9) {
         size_t avail = 0, total = 0;
         if (cudaMemGetInfo(&avail, &total) != cudaSuccess) {
